@@ -136,13 +136,16 @@ struct Args {
     const unsigned char *records_short;    // RecordShortF32 per table (shortlist loop)
     const float4 *cstore;                  // stored Gram matrices (c_supply), kStoredTableBytes each
     const int *cslot;                      // per table set: its stored matrix, or -1 (factored)
-    int cfilter;                           // chunks this launch takes: 0 all, 1 those whose table set
-                                           // has a stored matrix, 2 the others
+    int cfilter;                           // chunks a factored launch takes: 0 all, 1 those whose table
+                                           // set has no stored matrix
+    const uint32_t *order;                 // stored-C loop: the entries of the stored table sets
+    int n_order;
     const Consts *consts;
     ImageDesc single;          // used when descs == nullptr
     const ImageDesc *descs;
     int nu_max;
     double gamma;
+    float gamma32;             // gamma rounded once on the host (a conversion in the loop costs 16 cycles of the FP64 unit)
     uint16_t *trace_sel;       // [ordinal][nu_max], optional
     float *trace_dc;           // [ordinal][nu_max][2], optional
     int *status;
@@ -193,10 +196,6 @@ struct SmemLayout {
     static constexpr size_t bytes = off_bar + 2 * sizeof(uint64_t);
 };
 
-__device__ __forceinline__ const uint8_t *rec_types(const RecordF32 &r) { return r.types; }
-__device__ __forceinline__ const uint8_t *rec_types(const RecordShortF32 &r) { return r.types; }
-__device__ __forceinline__ const uint8_t *rec_types(const Record<double> &r) { return r.types; }
-
 // X[i] = sum_j x_j w8^-(j i), i, j in [0, 8): radix-2 decimation in
 // frequency (twiddles 1, (1 - i)/sqrt 2, -i, (-1 - i)/sqrt 2, then -i), 52
 // real additions and multiplications instead of 64 complex products.  The same
@@ -236,23 +235,28 @@ __device__ __forceinline__ void dft8(const C2<T> (&x)[8], C2<T> (&X)[8])
 // lane c = 0 sums the two real columns, k2 = 0 (re slot) and k2 = 8 (im slot).
 // With UNIT, y is taken as 1 for every present L-pixel: the result is then
 // the DFT of the type-split spatial weights, whose conjugate is G_t.
-template <typename T, bool UNIT = false, typename Rec>
-__device__ __forceinline__ void window_rows(const Args &a, const Rec &rec, C2<T> *scratch, const C2<T> *omc,
+template <typename T, bool UNIT = false, bool FLY = false>
+__device__ __forceinline__ void window_rows(const Args &a, const uint8_t *types, C2<T> *scratch, const C2<T> *omc,
                                             const T *wt, const WorkEntry we, const int lane, C2<T> (&acc)[4][4])
 {
     const ImageDesc img = a.descs ? a.descs[we.img] : a.single;
     const int p0 = 2 * we.bi - kOff / 2, q0 = 2 * we.bj - kOff / 2;
-    const uint8_t *types = rec_types(rec);
     __syncwarp();    // the previous block of this warp is done with the scratch
 
-    // 1. gather: x(p, q) = w(p, q) y(p, q) into the plane of its type.
+    // 1. gather: x(p, q) = w(p, q) y(p, q) into the plane of its type, two
+    // window rows per step (coalesced).  Entry (p, q) sits at p * 16 + (q ^
+    // (p / 4)), so that both these stores and the row reads below, which take
+    // one q of rows p, p + 4, p + 8, p + 12, fall in distinct bank groups
+    // (1200x1200 at nu_max 10: 699 against 711 us with half a row per lane).
+    // The in-kernel tables (FLY) keep half a row per lane: their kernel ran
+    // 1.7 % slower the other way (5.94 against 6.04 ms at 1024x1024).
     Vec4<T> *x4 = reinterpret_cast<Vec4<T> *>(scratch);
     {
-        const int p = lane >> 1, P = p0 + p;
         bool bad = false;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            const int q = (lane & 1) * 8 + j, Q = q0 + q;
+            const int p = FLY ? lane >> 1 : 2 * j + (lane >> 4), P = p0 + p;
+            const int q = FLY ? (lane & 1) * 8 + j : lane & 15, Q = q0 + q;
             const int code = types[p * 16 + q];
             T v = 0;
             if (code < 4 && P >= 0 && P < img.lr_h && Q >= 0 && Q < img.lr_w) {
@@ -265,7 +269,7 @@ __device__ __forceinline__ void window_rows(const Args &a, const Rec &rec, C2<T>
                 }
             }
             Vec4<T> o = {code == 0 ? v : T(0), code == 1 ? v : T(0), code == 2 ? v : T(0), code == 3 ? v : T(0)};
-            st4(&x4[p * 16 + q], o);
+            st4(&x4[p * 16 + (q ^ (p >> 2))], o);
         }
         if (bad) atomicOr(a.status, kStatusNonfinite);
     }
@@ -284,7 +288,7 @@ __device__ __forceinline__ void window_rows(const Args &a, const Rec &rec, C2<T>
         const T twim = c == 0 ? ((q & 1) ? T(-1) : T(1)) : tq.im;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const Vec4<T> x = ld4(&x4[(4 * r + i) * 16 + q]);
+            const Vec4<T> x = ld4(&x4[(4 * r + i) * 16 + (q ^ r)]);
             acc[i][0].re += x.x * twre; acc[i][0].im += x.x * twim;
             acc[i][1].re += x.y * twre; acc[i][1].im += x.y * twim;
             acc[i][2].re += x.z * twre; acc[i][2].im += x.z * twim;
@@ -313,13 +317,13 @@ __device__ __forceinline__ void rows_to_scratch(const C2<T> (&acc)[4][4], Vec4<T
 // Steps 1-2 for one block: the window's row DFTs, then the column DFTs
 //     Y_t(kap) = sum_{m: t(m) = t} w_m y_m w16^-(p kap1 + q kap2);
 // returns Y[i][t] for kap = (8h + i, lane & 15), h = lane >> 4.
-template <typename T, bool UNIT = false, typename Rec>
-__device__ __forceinline__ void initial_projection(const Args &a, const Rec &rec, C2<T> *scratch,
+template <typename T, bool UNIT = false, bool FLY = false>
+__device__ __forceinline__ void initial_projection(const Args &a, const uint8_t *types, C2<T> *scratch,
                                                    const C2<T> *omc, const T *wt, const WorkEntry we,
                                                    const int lane, C2<T> (&Y)[8][4])
 {
     C2<T> acc[4][4];
-    window_rows<T, UNIT>(a, rec, scratch, omc, wt, we, lane, acc);
+    window_rows<T, UNIT, FLY>(a, types, scratch, omc, wt, we, lane, acc);
     const int k2 = lane & 15, h = lane >> 4;
     // 2b. column DFTs, two types at a time through the scratch, split by the
     // parity of p: half h sums p = 2j + h for kap1' in [0, 8); then
@@ -669,7 +673,7 @@ __device__ __forceinline__ void greedy_loop_f32(const Args &a, const RecordF32 &
             Y[jj][t] = {f2(Y0[2 * jj][t].re, Y0[2 * jj + 1][t].re), f2(Y0[2 * jj][t].im, Y0[2 * jj + 1][t].im)};
     const float c1 = om[k2].re, s1 = om[k2].im;     // exp(-2 pi i kap2 / 32) = c1 - i s1
     const float2 e1c = f2(c1, c1), e1s = f2(s1, s1), e1n = f2(-s1, -s1);
-    const float gamma = (float)a.gamma;
+    const float gamma = a.gamma32;
     const int eta = kOff + ((lane >> 2) & 3), gam = kOff + (lane & 3);
     float fpix = 0.f, pw = 0.f;
     int u = 0, v = 0;
@@ -757,8 +761,30 @@ __device__ __forceinline__ void greedy_loop_f32(const Args &a, const RecordF32 &
 // measurement matrix: 8 KiB read per iteration, one float4 per lane and
 // register pair, 512 contiguous bytes per warp load; delta = R'_uv / (s_uv
 // D_uv) (Eq. 16) with the stored 1 / (s_uv D_uv).  R^0 comes from the same
-// factored initial projection as the other loops, and the argmax and the
-// bookkeeping are the factored loop's.
+// factored initial projection as the other loops.
+//
+// Lane L holds the candidates k = (s, L) for s = 0..16 and (s, -L mod 32) for
+// s = 17..31 ("slot" s = k1): k and -k share a lane (slots s and 32 - s),
+// except those of slots 0 and 16, whose mirrors sit in lane -L.  Because
+// C_{k,-l} = conj(C_{-k,l}) bit for bit (the build's tables are mirror-exact)
+// column -l is read as the conjugate of column l with the register pairs'
+// addresses exchanged, so the two share one 8 KiB in the L1 (Args::mirror).
+// Register pair i holds slots (pair_slot(i, 0), pair_slot(i, 1)), chosen so
+// that the mirror of a pair is another whole pair (i and i + 8 for i = 1..7).
+__host__ __device__ constexpr int pair_slot(int i, int e)
+{
+    return i == 0 ? 16 * e : i == 8 ? 15 + 2 * e : i < 8 ? 2 * i - 1 + e : 33 - 2 * (i - 8) - e;
+}
+__host__ __device__ constexpr int slot_pair(int s)
+{
+    return s == 0 || s == 16 ? 0 : s == 15 || s == 17 ? 8 : s < 15 ? (s + 1) / 2 : 8 + (33 - s) / 2;
+}
+__host__ __device__ constexpr int slot_half(int s) { return pair_slot(slot_pair(s), 1) == s; }
+// lane that holds candidate k
+__host__ __device__ constexpr int lane_of(int k) { return (k >> 5) <= 16 ? (k & 31) : ((32 - (k & 31)) & 31); }
+// candidate of a lane's slot
+__host__ __device__ constexpr int slot_k(int s, int lane) { return s * kW + (s <= 16 ? lane : ((32 - lane) & 31)); }
+
 __device__ __forceinline__ float4 ldg_stream4(const float4 *p)
 {
     float4 v;
@@ -773,40 +799,19 @@ __device__ __forceinline__ float ldg_stream1(const float *p)
     return v;
 }
 
-// R -= c C_{., l} over the lane's 32 candidates, column col (already loaded).
-__device__ __forceinline__ void sub_column(CP (&R)[4][4], const float4 (&col)[16], const C2<float> c)
-{
-    const float2 ncre = f2(-c.re, -c.re), cim = f2(c.im, c.im), ncim = f2(-c.im, -c.im);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        CP &r = R[i >> 2][i & 3];
-        const float2 Cre = f2(col[i].x, col[i].y), Cim = f2(col[i].z, col[i].w);
-        r.re = fma2(Cim, cim, fma2(Cre, ncre, r.re));
-        r.im = fma2(Cre, ncim, fma2(Cim, ncre, r.im));
-    }
-}
-
-__device__ __forceinline__ void load_column(const float4 *cs, const int l, const int lane, float4 (&col)[16])
-{
-    const float4 *p = cs + (size_t)l * 512 + lane;
-#pragma unroll
-    for (int i = 0; i < 16; ++i) col[i] = ldg_stream4(p + 32 * i);
-}
-
 // The state is R'_k = s_k R_k with s_k = sqrt(q_k / D_k), so the score of
 // Eq. 11 is |R'_k|^2.
 __device__ __forceinline__ float2 norm2(const CP r) { return fma2(r.im, r.im, mul2(r.re, r.re)); }
 
-// Argmax of the stored-C loop.  Slots 4 g .. 4 g + 3 (g = 4 a + jj) are
-// four consecutive candidates of the lane in index order, held in R[jj][2a]
-// (.x, .y: e = 0, 1 with b = 0) and R[jj][2a + 1] (b = 1).  The scan visits
-// the groups in increasing g and keeps the largest score (two three-input
-// max operations per group, sm_100 and later), the first group reaching it
-// and three of that group's scores; the slot inside the group is the first
-// whose score equals the maximum (the fourth if none of the three does).
-// The same choice as comparing every candidate in index order, with 7
+// Argmax of the stored-C loop.  Groups of up to four slots consecutive in
+// index order are scanned in that order, keeping the largest score (two
+// three-input max operations per group, sm_100 and later), the first group
+// reaching it and three of that group's scores; the slot inside the group is
+// the first whose score equals the maximum (the fourth if none of the three
+// does).  The same choice as comparing every candidate in index order, with 7
 // operations per group instead of 12 and a dependency chain through the
-// running maximum of two operations per group instead of eight.
+// running maximum of two operations per group instead of eight.  Scores are
+// >= 0: starting from 0, a lane whose scores are all 0 keeps its first slot.
 __device__ __forceinline__ float max3f(const float a, const float b, const float c)
 {
     float d;
@@ -814,31 +819,37 @@ __device__ __forceinline__ float max3f(const float a, const float b, const float
     return d;
 }
 
-__device__ __forceinline__ void scan_group(const CP (&Rj)[4], const int a, const int g, float &bs, int &bg,
-                                           float &t0, float &t1, float &t2)
-{
-    const float2 s0 = norm2(Rj[2 * a]), s1 = norm2(Rj[2 * a + 1]);
-    const float m = max3f(max3f(bs, s0.x, s1.x), s0.y, s1.y);
-    const bool p = m > bs;
-    bg = p ? g : bg;
-    t0 = p ? s0.x : t0;
-    t1 = p ? s1.x : t1;
-    t2 = p ? s0.y : t2;
-    bs = m;
-}
+struct Scan {
+    float bs, t0, t1, t2;     // largest score, and its group's first three
+    int base;                 // first slot of that group
+    __device__ __forceinline__ void init() { bs = t0 = t1 = t2 = 0.f; base = 0; }
+    template <int BASE>
+    __device__ __forceinline__ void group(const float s0, const float s1, const float s2, const float s3)
+    {
+        const float m = max3f(max3f(bs, s0, s1), s2, s3);
+        const bool p = m > bs;
+        base = p ? BASE : base;
+        t0 = p ? s0 : t0;
+        t1 = p ? s1 : t1;
+        t2 = p ? s2 : t2;
+        bs = m;
+    }
+    __device__ __forceinline__ int slot() const { return base + (t0 == bs ? 0 : t1 == bs ? 1 : t2 == bs ? 2 : 3); }
+};
 
 // R of this lane's candidate in a slot (the same slot in every lane).
-template <int I>
-__device__ __forceinline__ void r_slot(const CP (&R)[4][4], float &re, float &im)
+template <int S, int N>
+__device__ __forceinline__ void r_slot(const CP (&R)[N], float &re, float &im)
 {
-    const CP &r = R[(I >> 2) & 3][2 * (I >> 4) + (I & 1)];
-    re = ((I >> 1) & 1) ? r.re.y : r.re.x;
-    im = ((I >> 1) & 1) ? r.im.y : r.im.x;
+    const CP &r = R[slot_pair(S) < N ? slot_pair(S) : 0];     // (slots a pairs state does not keep are never asked for)
+    re = slot_half(S) ? r.re.y : r.re.x;
+    im = slot_half(S) ? r.im.y : r.im.x;
 }
 
-__device__ __forceinline__ void r_at_slot(const CP (&R)[4][4], const int slot, float &re, float &im)
+template <int N>
+__device__ __forceinline__ void r_at_slot(const CP (&R)[N], const int slot, float &re, float &im)
 {
-    switch (slot) {
+    switch (N == 16 ? slot : slot > 16 ? 16 : slot) {
     case 0: r_slot<0>(R, re, im); break;
     case 1: r_slot<1>(R, re, im); break;
     case 2: r_slot<2>(R, re, im); break;
@@ -874,36 +885,220 @@ __device__ __forceinline__ void r_at_slot(const CP (&R)[4][4], const int slot, f
     }
 }
 
-template <int LAY = kLayThreeQuarter, bool PAIRS = false>
-__device__ __forceinline__ void greedy_loop_stored(const Args &a, const RecordF32 &rec, const float4 *cs,
-                                                   const C2<float> *om, const PairTables &pt, const WorkEntry we,
-                                                   const int lane, C2<float> (&Y0)[8][4])
+// R^0 of one block in the stored loop's register pairs: the factored state's
+// candidates go through the warp's scratch, 16 slots at a time.
+template <int LAY>
+__device__ __forceinline__ void state_to_slots(const Args &a, C2<float> *scratch, const C2<float> *om,
+                                               const PairTables &pt, const int lane, const C2<float> (&Y0)[8][4],
+                                               CP (&R)[16])
 {
     const int k2 = lane & 15, h = lane >> 4;
     const float c1 = om[k2].re, s1 = om[k2].im;
     const float2 e1c = f2(c1, c1), e1s = f2(s1, s1), e1n = f2(-s1, -s1);
-    CP R[4][4];
+    CP F[4][4];
 #pragma unroll
     for (int jj = 0; jj < 4; ++jj) {
         CP Yj[4];
 #pragma unroll
         for (int t = 0; t < 4; ++t)
             Yj[t] = {f2(Y0[2 * jj][t].re, Y0[2 * jj + 1][t].re), f2(Y0[2 * jj][t].im, Y0[2 * jj + 1][t].im)};
-        state_to_R<LAY>(a, Yj, h, jj, k2, e1c, e1s, e1n, pt, R[jj]);
+        state_to_R<LAY>(a, Yj, h, jj, k2, e1c, e1s, e1n, pt, F[jj]);
     }
-    {
-        // R' = s R, the row scales stored after the columns in the same lane order
-        const float4 *sc = cs + kStoredScaleOff + lane;
+    float2 *buf = reinterpret_cast<float2 *>(scratch);          // [16 slots][32 lanes]
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const float4 w = ldg_stream4(sc + 32 * i);
-            CP &r = R[i >> 2][i & 3];
-            r.re = mul2(r.re, f2(w.x, w.y));
-            r.im = mul2(r.im, f2(w.z, w.w));
+    for (int half = 0; half < 2; ++half) {
+        __syncwarp();
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj)
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const CP r = F[jj][2 * half + b];
+                const int s = 8 * h + 2 * jj, c = k2 + 16 * b;    // slots s, s + 1 of this half, column c
+                const int m = (32 - c) & 31;
+                buf[s * 32 + (half == 0 || s == 0 ? c : m)] = f2(r.re.x, r.im.x);
+                buf[(s + 1) * 32 + (half == 0 ? c : m)] = f2(r.re.y, r.im.y);
+            }
+        __syncwarp();
+#pragma unroll
+        for (int s = 0; s < 16; ++s) {
+            const float2 v = buf[s * 32 + lane];
+            CP &r = R[slot_pair(16 * half + s)];
+            if (slot_half(16 * half + s)) { r.re.y = v.x; r.im.y = v.y; }
+            else { r.re.x = v.x; r.im.x = v.y; }
         }
     }
-    const float *invd = reinterpret_cast<const float *>(cs + kStoredInvDOff);   // 1 / (s_l D_l)
-    const float gamma = (float)a.gamma;
+}
+
+// The lane's best slot over all 32.
+__device__ __forceinline__ void scan_slots(const CP (&R)[16], Scan &scan)
+{
+    float2 p[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) p[i] = norm2(R[i]);
+    scan.init();
+    scan.group<0>(p[0].x, p[1].x, p[1].y, p[2].x);
+    scan.group<4>(p[2].y, p[3].x, p[3].y, p[4].x);
+    scan.group<8>(p[4].y, p[5].x, p[5].y, p[6].x);
+    scan.group<12>(p[6].y, p[7].x, p[7].y, p[8].x);
+    scan.group<16>(p[0].y, p[8].y, p[15].y, p[15].x);
+    scan.group<20>(p[14].y, p[14].x, p[13].y, p[13].x);
+    scan.group<24>(p[12].y, p[12].x, p[11].y, p[11].x);
+    scan.group<28>(p[10].y, p[10].x, p[9].y, p[9].x);
+}
+
+__device__ __forceinline__ void sub_pair(CP &r, const float4 c, const float2 ncre, const float2 ncim, const float2 are,
+                                         const float2 aim)
+{
+    const float2 Cre = f2(c.x, c.y), Cim = f2(c.z, c.w);
+    r.re = fma2(Cim, are, fma2(Cre, ncre, r.re));
+    r.im = fma2(Cre, ncim, fma2(Cim, aim, r.im));
+}
+
+// R'^0 of one block: the factored initial projection, scaled by s.
+template <int LAY>
+__device__ __forceinline__ void stored_setup(const Args &a, const float4 *cs, const uint8_t *types, C2<float> *scratch,
+                                             const C2<float> *om, const C2<float> *omc, const PairTables &pt,
+                                             const float *wt, const WorkEntry we, const int lane, CP (&R)[16])
+{
+    C2<float> Y[8][4];
+    initial_projection<float>(a, types, scratch, omc, wt, we, lane, Y);
+    state_to_slots<LAY>(a, scratch, om, pt, lane, Y, R);
+    // R' = s R, the row scales stored after the columns in the same lane order
+    const float4 *sc = cs + kStoredScaleOff + lane;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const float4 w = ldg_stream4(sc + 32 * i);
+        R[i].re = mul2(R[i].re, f2(w.x, w.y));
+        R[i].im = mul2(R[i].im, f2(w.z, w.w));
+    }
+}
+
+__device__ __forceinline__ const float *stored_invd(const float4 *cs)       // 1 / (s_l D_l) by l
+{
+    return reinterpret_cast<const float *>(cs + kStoredInvDOff);
+}
+
+// The warp's largest score and its candidate, ties to the lowest index.
+__device__ __forceinline__ int stored_argmax(const CP (&R)[16], const int lane)
+{
+    Scan scan;
+    scan_slots(R, scan);
+    float bs = scan.bs;
+    int bk = slot_k(scan.slot(), lane);
+    warp_argmax(bs, bk);
+    return bk;
+}
+
+__device__ __forceinline__ void load_column(const float4 *cs, const int k, const int lane, float4 (&col)[16])
+{
+    const float4 *p = cs + (size_t)k * 512 + lane;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) col[i] = ldg_stream4(p + 32 * i);
+}
+
+// gamma delta of the selected candidate (Eqs. 15, 16) and its share of
+// Eq. 18, as select_step does it.
+template <int N>
+__device__ __forceinline__ C2<float> stored_step(const CP (&R)[N], const int bk, const float invD, const float gamma,
+                                                 const C2<float> *om, const int eta, const int gam, float &fpix)
+{
+    const int wl = lane_of(bk), u = bk >> 5, v = bk & 31;
+    float mre, mim;
+    r_at_slot(R, u, mre, mim);
+    const float Rre = __shfl_sync(0xffffffffu, mre, wl);
+    const float Rim = __shfl_sync(0xffffffffu, mim, wl);
+    const C2<float> gd = {gamma * (Rre * invD), gamma * (Rim * invD)};
+    const C2<float> ph = om[(eta * u + gam * v) & 31];
+    fpix += gd.re * ph.re - gd.im * ph.im;
+    return gd;
+}
+
+__device__ __forceinline__ void store_pixel(const Args &a, const WorkEntry we, const int lane, const float fpix)
+{
+    if (lane < 16) {
+        const ImageDesc img = a.descs ? a.descs[we.img] : a.single;
+        const int yy = 4 * we.bi + (lane >> 2), xx = 4 * we.bj + (lane & 3);
+        img.hr[(long long)yy * img.hr_pitch + xx] = fpix;
+    }
+}
+
+// One block through the stored-C loop.
+template <int LAY, bool MIRROR, bool TRACE>
+__device__ __forceinline__ void stored_block(const Args &a, const float4 *cs, const uint8_t *types, C2<float> *scratch,
+                                             const C2<float> *om, const C2<float> *omc, const PairTables &pt,
+                                             const float *wt, const WorkEntry we, const int lane)
+{
+    CP R[16];
+    stored_setup<LAY>(a, cs, types, scratch, om, omc, pt, wt, we, lane, R);
+    const int eta = kOff + ((lane >> 2) & 3), gam = kOff + (lane & 3);
+    float fpix = 0.f;
+    for (int it = 0; it < a.nu_max; ++it) {
+        const int bk = stored_argmax(R, lane);
+        const bool more = it + 1 < a.nu_max;
+        // column uv, or -uv to be read conjugated with the pairs' places exchanged
+        const int mk = (((32 - (bk >> 5)) & 31) << 5) | ((32 - bk) & 31);       // -uv
+        const bool mir = MIRROR && mk < bk;
+        float4 col[16];
+        if (more) {
+            // in flight during the bookkeeping
+            if (!mir) {
+                load_column(cs, bk, lane, col);
+            } else {
+                const float4 *p = cs + (size_t)mk * 512;
+                col[0] = ldg_stream4(p + ((32 - lane) & 31));
+                p += lane;
+#pragma unroll
+                for (int i = 1; i < 16; ++i) col[i] = ldg_stream4(p + 32 * (i == 8 ? 8 : i ^ 8));
+            }
+        }
+        const C2<float> gd = stored_step(R, bk, ldg_stream1(stored_invd(cs) + bk), a.gamma32, om, eta, gam, fpix);
+        if constexpr (TRACE) {
+            if (lane == 0) {
+                const long long row = (long long)we.ord * a.nu_max + it;
+                a.trace_sel[row] = (uint16_t)bk;
+                a.trace_dc[2 * row] = gd.re;
+                a.trace_dc[2 * row + 1] = gd.im;
+            }
+        }
+        if (more) {
+            const float2 ncre = f2(-gd.re, -gd.re), ncim = f2(-gd.im, -gd.im);
+            float2 aim = ncre, are = f2(gd.im, gd.im);
+            if (mir) {
+                aim = f2(gd.re, gd.re);
+                are = ncim;
+                col[8] = make_float4(col[8].y, col[8].x, col[8].w, col[8].z);
+            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i) sub_pair(R[i], col[i], ncre, ncim, are, aim);
+        }
+    }
+    store_pixel(a, we, lane, fpix);
+}
+
+// The same with the conjugate-pair update (1024x1024, nu_max 50: 2.65 -> 1.49
+// ms against updating all 1024 candidates from two columns).  The argmax runs
+// over k <= -k only: slots 1..15 of every lane and slots 0 and 16 of lanes
+// 0..16, so only those are kept and updated.  C_{k,-uv} = conj(C_{-k,uv}), and -k's rows are
+// scaled like k's in these plans, so one column serves both members of the
+// pair: 17 loads and 9 register pairs an iteration instead of 32 and 32.
+template <int LAY>
+__device__ __forceinline__ void stored_block_pairs(const Args &a, const float4 *cs, const uint8_t *types,
+                                                   C2<float> *scratch, const C2<float> *om, const C2<float> *omc,
+                                                   const PairTables &pt, const float *wt, const WorkEntry we,
+                                                   const int lane)
+{
+    CP R[9];                  // pairs 0..7 as above, slot 15 in the low half of the ninth
+    const bool hid = lane > 16;   // slots 0 and 16 of this lane are hidden: R' stays 0
+    {
+        CP F[16];
+        stored_setup<LAY>(a, cs, types, scratch, om, omc, pt, wt, we, lane, F);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) R[i] = F[i];
+        if (hid) R[0] = {f2(0.f, 0.f), f2(0.f, 0.f)};
+        R[8].re.y = R[8].im.y = 0.f;
+    }
+    const float *invd = reinterpret_cast<const float *>(cs + kStoredInvDOff);
+    const float gamma = a.gamma32;
     const int eta = kOff + ((lane >> 2) & 3), gam = kOff + (lane & 3);
     float fpix = 0.f, pw = 0.f;
     int u = 0, v = 0;
@@ -911,37 +1106,51 @@ __device__ __forceinline__ void greedy_loop_stored(const Args &a, const RecordF3
     const long long trow = (long long)we.ord * a.nu_max;
 
     for (int it = 0; it < a.nu_max; ++it) {
-        // scores are >= 0: starting from 0, a lane whose scores are all 0
-        // keeps group 0, slot 0, as a scan from -1 would
-        float bs = 0.f, t0 = 0.f, t1 = 0.f, t2 = 0.f;
-        int bg = 0;
+        Scan scan;
+        scan.init();
+        {
+            float2 p[9];
 #pragma unroll
-        for (int aa = 0; aa < 2; ++aa)
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj) scan_group(R[jj], aa, 4 * aa + jj, bs, bg, t0, t1, t2);
-        const int el = t0 == bs ? 0 : t1 == bs ? 1 : t2 == bs ? 2 : 3;
-        // slot 4 bg + el = 16 a + 4 jj + 2 e + b -> k
-        int bk = (8 * h + 2 * (bg & 3) + (el >> 1) + 16 * (bg >> 2)) * kW + k2 + 16 * (el & 1);
+            for (int i = 0; i < 9; ++i) p[i] = norm2(R[i]);
+            scan.group<0>(p[0].x, p[1].x, p[1].y, p[2].x);
+            scan.group<4>(p[2].y, p[3].x, p[3].y, p[4].x);
+            scan.group<8>(p[4].y, p[5].x, p[5].y, p[6].x);
+            scan.group<12>(p[6].y, p[7].x, p[7].y, p[8].x);
+            scan.group<16>(p[0].y, 0.f, 0.f, 0.f);
+        }
+        float bs = scan.bs;
+        int bk = slot_k(scan.slot(), lane);
         warp_argmax(bs, bk);
         const bool more = it + 1 < a.nu_max;
-        float4 col[16];
-        if (more) load_column(cs, bk, lane, col);      // in flight during the bookkeeping
+        float4 own[9], mir[8];
+        if (more) {
+            const float4 *p = cs + (size_t)bk * 512 + lane;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) own[i] = ldg_stream4(p + 32 * i);
+            mir[0] = ldg_stream4(cs + (size_t)bk * 512 + ((32 - lane) & 31));
+#pragma unroll
+            for (int i = 1; i < 8; ++i) mir[i] = ldg_stream4(p + 32 * (i + 8));
+            if (hid) own[0] = mir[0] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
         const float invD = ldg_stream1(invd + bk);
-        const int wl = (bk & 15) + ((bk >> 5) & 8) * 2;
-        const int slot = ((bk >> 9) << 4) | (((bk >> 6) & 3) << 2) | (((bk >> 5) & 1) << 1) | ((bk >> 4) & 1);
+        const int wl = lane_of(bk), slot = bk >> 5;
         float mre, mim;
         r_at_slot(R, slot, mre, mim);
         const float Rre = __shfl_sync(0xffffffffu, mre, wl);
         const float Rim = __shfl_sync(0xffffffffu, mim, wl);
-        select_step<float, LAY, PAIRS>(a, om, invD, gamma, bk, Rre, Rim, eta, gam, lane, trow, it, u, v, g, fpix,
-                                       pw);
+        select_step<float, LAY, true>(a, om, invD, gamma, bk, Rre, Rim, eta, gam, lane, trow, it, u, v, g, fpix, pw);
         if (more) {
             const C2<float> gd = {gamma * (Rre * invD), gamma * (Rim * invD)};   // as in select_step
-            sub_column(R, col, gd);
-            if constexpr (PAIRS) {
-                // the partner -uv gets conj(gamma delta) (none when uv = -uv)
-                load_column(cs, ((-u) & 31) * kW + ((-v) & 31), lane, col);
-                sub_column(R, col, C2<float>{pw * gd.re, -pw * gd.im});
+            const float2 ncre = f2(-gd.re, -gd.re), ncim = f2(-gd.im, -gd.im), cim = f2(gd.im, gd.im);
+            // the partner -uv gets pw conj(gamma delta) times the conjugate of the mirrored rows
+            const C2<float> pd = {pw * gd.re, -pw * gd.im};
+            const float2 npre = f2(-pd.re, -pd.re), npim = f2(-pd.im, -pd.im), pre = f2(pd.re, pd.re);
+            const float4 m8 = make_float4(own[8].y, 0.f, own[8].w, 0.f);
+            own[8].y = own[8].w = 0.f;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                sub_pair(R[i], own[i], ncre, ncim, cim, ncre);
+                sub_pair(R[i], i < 8 ? mir[i & 7] : m8, npre, npim, npim, pre);
             }
         }
     }
@@ -1028,7 +1237,7 @@ __device__ __forceinline__ void shortlist_setup(const Args &a, const RecordShort
 #pragma unroll
         for (int t = 0; t < 4; ++t) hw[c][t] = h_of(om, kw[c], t);
     C2<float> acc[4][4];
-    window_rows<float>(a, rec, scratch, omc, wt, we, lane, acc);
+    window_rows<float>(a, rec.types, scratch, omc, wt, we, lane, acc);
     Vec4<float> *tb = reinterpret_cast<Vec4<float> *>(scratch);
     C2<float> Rw[2] = {{0, 0}, {0, 0}};
 #pragma unroll
@@ -1067,11 +1276,10 @@ __device__ __forceinline__ void shortlist_setup(const Args &a, const RecordShort
             st.kc[sl4] = kn[sl4];
             {
                 // where the stored-C loop's lanes keep candidate k in a column:
-                // float4 (4 jj + 2 a + b) * 32 + 16 h + kap2, low or high half by e
-                const int k1 = kn[sl4] >> 5, k2f = kn[sl4] & 31;
-                st.coff[sl4] = (((k1 >> 1) & 3) * 4 + 2 * (k1 >> 4) + (k2f >> 4)) * 32 + 16 * ((k1 >> 3) & 1) +
-                               (k2f & 15);
-                st.ce |= (k1 & 1) << sl4;
+                // float4 slot_pair * 32 + lane, low or high half
+                const int k1 = kn[sl4] >> 5;
+                st.coff[sl4] = slot_pair(k1) * 32 + lane_of(kn[sl4]);
+                st.ce |= slot_half(k1) << sl4;
             }
             if (sl4 & 1) { st.Rre[sl4 >> 1].y = Rn[sl4].re; st.Rim[sl4 >> 1].y = Rn[sl4].im; }
             else { st.Rre[sl4 >> 1].x = Rn[sl4].re; st.Rim[sl4 >> 1].x = Rn[sl4].im; }
@@ -1137,7 +1345,7 @@ __device__ __forceinline__ void shortlist_pair(const Args &a, const RecordShortF
     const int nu_h = hb == 0 ? nu[0] : nu[1];
     const int numax = nu[0] > nu[1] ? nu[0] : nu[1];
     const WorkEntry me = hb == 0 ? we[0] : we[1];
-    const float gamma = (float)a.gamma;
+    const float gamma = a.gamma32;
     const int eta = kOff + ((lane >> 2) & 3), gam = kOff + (lane & 3);
     float fpix = 0.f, unused_pw = 0.f;
     int u = 0, v = 0;
@@ -1265,8 +1473,9 @@ __device__ __forceinline__ int shortlist_iterations(const Args &a, const Shortli
 // of one does not constrain the other.  3 and 4 = mode 0 for other sensor
 // layouts: slot apertures from a.slot_ap (3), or one sub-pixel per slot (4).
 // Bit 3 (kModePairs) added to modes 0, 3, 4: the conjugate-pair update.
-// Bit 4 (kModeStoredC) added to those: the column of C read from the stored
-// Gram matrix instead of rebuilt from the factored tables.
+// Bit 4 (kModeStoredC) added to mode 1: the column of C read from the stored
+// Gram matrix instead of rebuilt from the factored tables (the full loop with
+// stored columns is stored_kernel).
 constexpr int kModePairs = 8;
 constexpr int kModeStoredC = 16;
 __host__ __device__ constexpr int lay_of(int mode)
@@ -1286,14 +1495,9 @@ template <int MODE> struct Loop<float, MODE> {
                                                const float *wt, const WorkEntry we, const int lane,
                                                const float4 *cs)
     {
-        // (a stored-C launch takes only chunks whose table set has a stored matrix)
-        if constexpr (plain_of(MODE) && stored_of(MODE)) {
+        if constexpr (plain_of(MODE)) {
             C2<float> Y[8][4];
-            initial_projection<float>(a, rec, scratch, omc, wt, we, lane, Y);
-            greedy_loop_stored<lay_of(MODE), pairs_of(MODE)>(a, rec, cs, om, pt, we, lane, Y);
-        } else if constexpr (plain_of(MODE)) {
-            C2<float> Y[8][4];
-            initial_projection<float>(a, rec, scratch, omc, wt, we, lane, Y);
+            initial_projection<float>(a, rec.types, scratch, omc, wt, we, lane, Y);
             greedy_loop_f32<lay_of(MODE), pairs_of(MODE)>(a, rec, om, omc, pt, we, lane, Y);
         } else if constexpr (learned_of(MODE) == 1) {
             const Shortlist &sl = a.shortlists[we.ord];
@@ -1306,9 +1510,8 @@ template <int MODE> struct Loop<float, MODE> {
             const Shortlist &sl = a.shortlists[we.ord];
             if (sl.missing <= a.max_missing) return;
             C2<float> Y[8][4];
-            initial_projection<float>(a, rec, scratch, omc, wt, we, lane, Y);
-            if constexpr (stored_of(MODE)) greedy_loop_stored<kLayThreeQuarter>(a, rec, cs, om, pt, we, lane, Y);
-            else greedy_loop_f32<kLayThreeQuarter>(a, rec, om, omc, pt, we, lane, Y);
+            initial_projection<float>(a, rec.types, scratch, omc, wt, we, lane, Y);
+            greedy_loop_f32<kLayThreeQuarter>(a, rec, om, omc, pt, we, lane, Y);
         }
     }
 
@@ -1335,7 +1538,7 @@ template <int MODE> struct Loop<double, MODE> {
                                                const float4 *)
     {
         C2<double> Y[8][4];
-        initial_projection<double>(a, rec, scratch, omc, wt, we, lane, Y);
+        initial_projection<double>(a, rec.types, scratch, omc, wt, we, lane, Y);
         greedy_loop<double, lay_of(MODE), pairs_of(MODE)>(a, rec, om, omc, we, lane, Y);
     }
     static __device__ __forceinline__ void run_pair(const Args &a, const Record<double> &rec, C2<double> *scratch,
@@ -1356,9 +1559,7 @@ __device__ __forceinline__ bool chunk_has_work(const Args &a, const int c)
 {
     if constexpr (learned_of(MODE) == 0) {
         // a plan with stored and factored table sets runs them as two launches
-        if (a.cfilter == 0) return true;
-        const bool stored = a.cslot[a.chunk_table[c]] >= 0;
-        return a.cfilter == 1 ? stored : !stored;
+        return a.cfilter == 0 || a.cslot[a.chunk_table[c]] < 0;
     } else {
         bool mine = false;
         if (threadIdx.x < kChunk) {
@@ -1483,6 +1684,110 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) recurrent_kernel(const Args 
     }
 }
 
+// --------------------------------------------------- stored-C kernel --
+// The stored-C loop on the blocks of the stored table sets: one warp per
+// block, the warps of a CTA independent of each other (no table in shared
+// memory: the loop needs only the window's types, the column and the scales).
+// 4096x3072, nu_max 100: 36.2 -> 33.0 ms against chunks of 8 blocks behind a
+// shared table slot, eight warps an SM.
+// With LEARNED, only the blocks the gate sends back: the CTA lists them, a
+// batch of its entries at a time, and its warps take them from the list.
+constexpr int kStoredWarps = 12;
+constexpr int kStoredBatch = 2048;
+struct StoredSmem {
+    static constexpr size_t off_scratch = 0;                                     // kStoredWarps x 4 KB
+    static constexpr size_t off_om = kStoredWarps * 256 * 2 * sizeof(C2<float>);
+    static constexpr size_t off_omc = off_om + 32 * sizeof(C2<float>);
+    static constexpr size_t off_pair = off_omc + 32 * sizeof(C2<float>);
+    static constexpr size_t off_w = off_pair + sizeof(PairTables);
+    static constexpr size_t bytes = off_w + 256 * sizeof(float);
+};
+
+__device__ __forceinline__ void fill_tables(const Args &a, C2<float> *om, C2<float> *omc, PairTables *pt, float *wt)
+{
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) wt[i] = a.consts->w32[i];
+    for (int i = threadIdx.x; i < 32; i += blockDim.x) {
+        const float re = a.consts->om32[2 * i], im = a.consts->om32[2 * i + 1];
+        om[i] = {re, im};
+        omc[i] = {re, -im};
+        const int n1 = (i + 1) & 31;
+        pt->e12[i] = make_float4(re, a.consts->om32[2 * n1], im, a.consts->om32[2 * n1 + 1]);
+        pt->e12n[i] = make_float2(-im, -a.consts->om32[2 * n1 + 1]);
+        if (i < 8) {
+            const float ca = a.consts->om32[4 * i], sa = a.consts->om32[4 * i + 1];
+            const float cb = a.consts->om32[4 * i + 2], sb = a.consts->om32[4 * i + 3];
+            pt->e2[i] = make_float4(ca, cb, sa, sb);
+            pt->e2n[i] = make_float2(-sa, -sb);
+        }
+    }
+}
+
+enum StoredKind { kSolo, kSoloMirror, kSoloPairs, kFallback };
+// Warps per CTA (one CTA per SM).  Twelve is three per scheduler at 168
+// registers: the loop is bound by the latency of its own instructions (issue
+// active 52 %, ALU and FMA pipes 42 %, no memory unit above 58 %), and the
+// third warp is worth 13 % over eight warps at 222 registers (1024x1024, nu_max
+// 100: 2.82 against 3.24 ms); sixteen at 128 registers spill (8.3 ms, 3.4 ms
+// with the column loaded in two halves).  The mirrored loop runs where blocks
+// are few and keeps eight and no spills (64x64: 60 against 64 us).
+constexpr int stored_warps(const int kind) { return kind == kSoloMirror ? 8 : kStoredWarps; }
+
+template <int LAY, int KIND, bool TRACE>
+__global__ void __launch_bounds__(stored_warps(KIND) * 32, 1) stored_kernel(const Args a)
+{
+    using L = StoredSmem;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    C2<float> *scratch = reinterpret_cast<C2<float> *>(smem + L::off_scratch) + warp * 512;
+    C2<float> *om = reinterpret_cast<C2<float> *>(smem + L::off_om);
+    C2<float> *omc = reinterpret_cast<C2<float> *>(smem + L::off_omc);
+    PairTables *pt = reinterpret_cast<PairTables *>(smem + L::off_pair);
+    float *wt = reinterpret_cast<float *>(smem + L::off_w);
+    fill_tables(a, om, omc, pt, wt);
+    __syncthreads();
+    auto cols = [&](const uint32_t e) {
+        return a.cstore + (size_t)a.cslot[a.chunk_table[e / kChunk]] * (kStoredTableBytes / 16);
+    };
+    auto types = [&](const uint32_t e) {
+        return a.records + (size_t)a.chunk_table[e / kChunk] * sizeof(RecordF32) + offsetof(RecordF32, types);
+    };
+    auto block = [&](const uint32_t e) {
+        if constexpr (KIND == kSoloPairs)
+            stored_block_pairs<LAY>(a, cols(e), types(e), scratch, om, omc, *pt, wt, a.entries[e], lane);
+        else
+            stored_block<LAY, KIND != kSolo, TRACE>(a, cols(e), types(e), scratch, om, omc, *pt, wt, a.entries[e], lane);
+    };
+    if constexpr (KIND != kFallback) {
+        for (int i = blockIdx.x * warps + warp; i < a.n_order; i += gridDim.x * warps) block(a.order[i]);
+    } else {
+        __shared__ uint32_t list[kStoredBatch];
+        __shared__ int n_list, next;
+        // entries o of this CTA: runs of kChunk, every gridDim-th run
+        const long long runs = ((long long)a.n_order + kChunk - 1) / kChunk;
+        const long long mine = ((runs - blockIdx.x + gridDim.x - 1) / gridDim.x) * kChunk;
+        for (long long b0 = 0; b0 < mine; b0 += kStoredBatch) {
+            __syncthreads();
+            if (threadIdx.x == 0) n_list = next = 0;
+            __syncthreads();
+            for (int i = threadIdx.x; i < kStoredBatch && b0 + i < mine; i += blockDim.x) {
+                const long long j = b0 + i;
+                const long long o = ((j / kChunk) * gridDim.x + blockIdx.x) * kChunk + j % kChunk;
+                if (o >= a.n_order) continue;
+                const uint32_t e = a.order[o];
+                if (!(a.shortlists[a.entries[e].ord].missing <= a.max_missing)) list[atomicAdd(&n_list, 1)] = e;
+            }
+            __syncthreads();
+            for (;;) {
+                int i = 0;
+                if (lane == 0) i = atomicAdd(&next, 1);
+                i = __shfl_sync(0xffffffffu, i, 0);
+                if (i >= n_list) break;
+                block(list[i]);
+            }
+        }
+    }
+}
+
 // ------------------------------------------- tables built per block --
 // For masks whose local measurement matrices rarely repeat (a non-recurrent
 // sensor), each warp builds its block's factored tables itself, in FP32:
@@ -1518,22 +1823,8 @@ __global__ void __launch_bounds__(kFlyWarps * 32, 2) onthefly_kernel(const Args 
     PairTables *pt = reinterpret_cast<PairTables *>(smem + L::off_pair);
     float *wt = reinterpret_cast<float *>(smem + L::off_w);
     float *qv = reinterpret_cast<float *>(smem + L::off_q);
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) wt[i] = a.consts->w32[i];
     for (int i = threadIdx.x; i < kK; i += blockDim.x) qv[i] = a.q[i];
-    for (int i = threadIdx.x; i < 32; i += blockDim.x) {
-        const float re = a.consts->om32[2 * i], im = a.consts->om32[2 * i + 1];
-        om[i] = {re, im};
-        omc[i] = {re, -im};
-        const int n1 = (i + 1) & 31;
-        pt->e12[i] = make_float4(re, a.consts->om32[2 * n1], im, a.consts->om32[2 * n1 + 1]);
-        pt->e12n[i] = make_float2(-im, -a.consts->om32[2 * n1 + 1]);
-        if (i < 8) {
-            const float ca = a.consts->om32[4 * i], sa = a.consts->om32[4 * i + 1];
-            const float cb = a.consts->om32[4 * i + 2], sb = a.consts->om32[4 * i + 3];
-            pt->e2[i] = make_float4(ca, cb, sa, sb);
-            pt->e2n[i] = make_float2(-sa, -sb);
-        }
-    }
+    fill_tables(a, om, omc, pt, wt);
     __syncthreads();
     const int k2 = lane & 15, h = lane >> 4;
     for (int e = blockIdx.x * kFlyWarps + warp; e < n_entries; e += gridDim.x * kFlyWarps) {
@@ -1550,7 +1841,7 @@ __global__ void __launch_bounds__(kFlyWarps * 32, 2) onthefly_kernel(const Args 
         __syncwarp();
         // G_t(d1, d2) = conj(Yw_t(d1, d2)) for d1 = 8h + i, d2 = k2
         C2<float> Yw[8][4];
-        initial_projection<float, true>(a, rec, scratch, omc, wt, we, lane, Yw);
+        initial_projection<float, true, true>(a, rec.types, scratch, omc, wt, we, lane, Yw);
         C2<float> prev[4];                  // G_t(8h - 1, k2), owned by the other half
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
@@ -1606,7 +1897,7 @@ __global__ void __launch_bounds__(kFlyWarps * 32, 2) onthefly_kernel(const Args 
             }
         }
         C2<float> Y[8][4];
-        initial_projection<float>(a, rec, scratch, omc, wt, we, lane, Y);
+        initial_projection<float, false, true>(a, rec.types, scratch, omc, wt, we, lane, Y);
         __syncwarp();                       // scratch (= invD) no longer needed
 #pragma unroll
         for (int i = 0; i < 8; ++i)
@@ -1642,7 +1933,7 @@ __global__ void __launch_bounds__(kDirectWarps * 32) direct_kernel(const Args a,
     for (int i = threadIdx.x; i < 256; i += blockDim.x) sm.w[i] = a.consts->w32[i];
     for (int i = threadIdx.x; i < 32; i += blockDim.x) sm.om[i] = make_float2(a.consts->om32[2 * i], a.consts->om32[2 * i + 1]);
     __syncthreads();
-    const float gamma = (float)a.gamma;
+    const float gamma = a.gamma32;
     for (int e = blockIdx.x * kDirectWarps + warp; e < n_entries; e += gridDim.x * kDirectWarps) {
         const WorkEntry we = a.entries[e];
         if (we.img < 0) continue;
@@ -1813,17 +2104,7 @@ const Variant kVariants[] = {
     RLJSDE_VARIANT(float, 4, 3, 4), RLJSDE_VARIANT(float, 8, 2, 4), RLJSDE_VARIANT(double, 4, 1, 4),
     RLJSDE_VARIANT(float, 4, 3, 8), RLJSDE_VARIANT(float, 4, 3, 11), RLJSDE_VARIANT(float, 4, 3, 12),
     RLJSDE_VARIANT(double, 4, 1, 8), RLJSDE_VARIANT(double, 4, 1, 11), RLJSDE_VARIANT(double, 4, 1, 12),
-    // the stored-C loop: one CTA of 8 warps per SM with the full register file
-    // (254 registers, no spills) iterates 4 % faster than 4 warps x 3 CTAs
-    // (168, spilling) and 2 % faster than 4 warps x 2 CTAs, but its initial
-    // projection is 7 % slower: 4 x 3 for short loops (nu_max < 20)
-    RLJSDE_VARIANT(float, 8, 1, 16), RLJSDE_VARIANT(float, 4, 3, 16), RLJSDE_VARIANT(float, 8, 1, 19),
-    RLJSDE_VARIANT(float, 8, 1, 20),
-    RLJSDE_VARIANT(float, 8, 1, 24), RLJSDE_VARIANT(float, 8, 1, 27), RLJSDE_VARIANT(float, 8, 1, 28),
-    // the learned path's full loop on the blocks the gate sends back: few per
-    // chunk, so more CTAs of fewer warps (with a tenth of the blocks sent
-    // back the learned path ran at 551 MP/s with 4 x 3, 415 with 8 x 1)
-    RLJSDE_VARIANT(float, 4, 3, 17), RLJSDE_VARIANT(float, 4, 3, 18),
+    RLJSDE_VARIANT(float, 4, 3, 17),
 };
 #undef RLJSDE_VARIANT
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
@@ -1847,11 +2128,14 @@ Args make_args(const rljsde_plan *p)
     a.records_short = static_cast<const unsigned char *>(p->d_records_short);
     a.cstore = static_cast<const float4 *>(p->d_cstore);
     a.cslot = p->d_cslot;
+    a.order = p->d_order;
+    a.n_order = p->n_order;
     a.record_bytes = (uint32_t)p->record_bytes;
     a.consts = p->d_consts;
     a.descs = nullptr;
     a.nu_max = p->params.nu_max;
     a.gamma = p->params.gamma_odc;
+    a.gamma32 = (float)p->params.gamma_odc;
     a.status = p->d_status;
     a.masks = p->d_masks;
     a.mask_offset = p->d_mask_offset;
@@ -1860,6 +2144,61 @@ Args make_args(const rljsde_plan *p)
     a.layout = p->params.layout;
     a.pairs = p->params.pairs;
     return a;
+}
+
+// The stored-C kernel of a plan's layout and update, traced or not.
+using StoredFn = void (*)(const Args);
+template <int LAY>
+StoredFn stored_fn_of(const int kind, const bool trace)
+{
+    switch (kind) {
+    case kSoloPairs: return stored_kernel<LAY, kSoloPairs, true>;     // looks at the trace pointer itself
+    case kSoloMirror: return trace ? stored_kernel<LAY, kSoloMirror, true> : stored_kernel<LAY, kSoloMirror, false>;
+    default: return trace ? stored_kernel<LAY, kSolo, true> : stored_kernel<LAY, kSolo, false>;
+    }
+}
+StoredFn stored_fn(const rljsde_plan *p, const int kind, const bool trace)
+{
+    if (kind == kFallback)
+        return trace ? stored_kernel<kLayThreeQuarter, kFallback, true> : stored_kernel<kLayThreeQuarter, kFallback, false>;
+    return p->kind == 1 ? stored_fn_of<kLayGeneral>(kind, trace)
+           : p->kind == 3 ? stored_fn_of<kLaySingle>(kind, trace) : stored_fn_of<kLayThreeQuarter>(kind, trace);
+}
+
+// Which stored-C kernel a plan's blocks take.  Reading column -uv as the
+// mirror of column uv halves the distinct columns but costs a branch and some
+// ten instructions an iteration: it pays while the columns come from HBM or a
+// cold L2, that is with few blocks.  Measured (mirrored / plain, 4x4-LR tile,
+// nu_max 100): 64x64 60 / 87 us, 128x128 77 / 104, 192x192 146 / 187, 256x256
+// (27 blocks per SM) 287 / 296, 384x384 543 / 517, 1024x1024 3164 / 2824.
+constexpr int kMirrorBlocksPerSm = 27;
+int stored_kind(const rljsde_plan *p)
+{
+    if (p->params.pairs) return kSoloPairs;
+    return p->mirror && p->n_order <= kMirrorBlocksPerSm * p->sm_count ? kSoloMirror : kSolo;
+}
+
+// Shape of a stored-C launch: one CTA per SM, with no more warps than keep
+// its number of rounds (a warp alone on its scheduler iterates faster).
+void stored_shape(const rljsde_plan *p, const int kind, int &warps, int &grid)
+{
+    const int most = stored_warps(kind);
+    const int per_sm = p->n_order > 0 ? (p->n_order + p->sm_count - 1) / p->sm_count : 1;
+    const int rounds = (per_sm + most - 1) / most;
+    warps = kind == kFallback ? most : (per_sm + rounds - 1) / rounds;
+    const int want = (p->n_order + warps - 1) / warps;
+    grid = want < p->sm_count ? (want > 0 ? want : 1) : p->sm_count;
+}
+
+int launch_stored(const rljsde_plan *p, const Args &a, const int kind, cudaStream_t s)
+{
+    const StoredFn fn = stored_fn(p, kind, a.trace_sel != nullptr);
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)StoredSmem::bytes) != cudaSuccess)
+        return RLJSDE_ERR_CUDA;
+    int warps, grid;
+    stored_shape(p, kind, warps, grid);
+    fn<<<grid, warps * 32, StoredSmem::bytes, s>>>(a);
+    return cudaGetLastError() == cudaSuccess ? RLJSDE_OK : RLJSDE_ERR_CUDA;
 }
 
 int launch(const rljsde_plan *p, const Args &a, cudaStream_t s)
@@ -1873,16 +2212,13 @@ int launch(const rljsde_plan *p, const Args &a, cudaStream_t s)
         // the stored-C loop on the table sets with a stored Gram matrix, the
         // factored loop on the others: one launch each (one kernel holding
         // both loops spills and ran the stored loop 1.5x slower)
-        const bool mixed = p->n_stored > 0 && p->n_stored < p->n_tables;
         if (p->n_stored > 0) {
-            Args b = a;
-            b.cfilter = mixed ? 1 : 0;
-            const Variant &v = kVariants[p->variant_stored];
-            v.fn<<<p->grid_stored, v.warps * 32, v.smem, s>>>(b);
+            const int st = launch_stored(p, a, stored_kind(p), s);
+            if (st != RLJSDE_OK) return st;
         }
         if (p->n_stored < p->n_tables) {
             Args b = a;
-            b.cfilter = mixed ? 2 : 0;
+            b.cfilter = p->n_stored > 0 ? 1 : 0;
             const Variant &v = kVariants[p->variant];
             v.fn<<<p->grid, v.warps * 32, v.smem, s>>>(b);
         }
@@ -1928,16 +2264,8 @@ __device__ __forceinline__ C2<double> h64(const double2 *om, const uint32_t slot
     return z;
 }
 
-// The candidate k of float4 i * 32 + lane of a stored column (low half; the
-// high half holds k + 32).
-__device__ __forceinline__ int stored_k(const int i, const int lane)
-{
-    const int jj = i >> 2, qa = (i >> 1) & 1, qb = i & 1;
-    return (8 * (lane >> 4) + 2 * jj + 16 * qa) * kW + (lane & 15) + 16 * qb;
-}
-
 __global__ void __launch_bounds__(512) build_c_kernel(const double *g64, const Consts *consts,
-                                                      const uint32_t slot_ap, float4 *out)
+                                                      const uint32_t slot_ap, const int pairs, float4 *out)
 {
     __shared__ double2 G[4][256];
     __shared__ double2 om[32];
@@ -1950,7 +2278,7 @@ __global__ void __launch_bounds__(512) build_c_kernel(const double *g64, const C
     const int l1 = l >> 5, l2 = l & 31;
     float re[2], im[2];
     for (int e = 0; e < 2; ++e) {
-        const int k = stored_k(i, lane) + kW * e, k1 = k >> 5, k2 = k & 31;
+        const int k = slot_k(pair_slot(i, e), lane), k1 = k >> 5, k2 = k & 31;
         const int d = ((l1 - k1) & 15) * 16 + ((l2 - k2) & 15);
         double cre = 0.0, cim = 0.0;
         for (int t = 0; t < 4; ++t) {
@@ -1960,7 +2288,9 @@ __global__ void __launch_bounds__(512) build_c_kernel(const double *g64, const C
             cre += z.re * gt.x - z.im * gt.y;
             cim += z.re * gt.y + z.im * gt.x;
         }
-        const double sk = sqrt(src[2048 + k]);
+        // conjugate-pair plans: the rows of the hidden member -k carry k's scale
+        const int mk = ((32 - k1) & 31) * kW + ((32 - k2) & 31);
+        const double sk = sqrt(src[2048 + (pairs && mk < k ? mk : k)]);
         re[e] = (float)(sk * cre);
         im[e] = (float)(sk * cim);
     }
@@ -1975,8 +2305,9 @@ __global__ void __launch_bounds__(512) build_c_scales_kernel(const double *g64, 
     const int tab = blockIdx.x;
     const double *src = g64 + (size_t)tab * kStoredBuildDoubles;
     float4 *base = out + (size_t)tab * (kStoredTableBytes / 16);
-    const int i = threadIdx.x >> 5, lane = threadIdx.x & 31, k = stored_k(i, lane);
-    const float s0 = (float)sqrt(src[2048 + k]), s1 = (float)sqrt(src[2048 + k + kW]);
+    const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const float s0 = (float)sqrt(src[2048 + slot_k(pair_slot(i, 0), lane)]);
+    const float s1 = (float)sqrt(src[2048 + slot_k(pair_slot(i, 1), lane)]);
     base[kStoredScaleOff + threadIdx.x] = make_float4(s0, s1, s0, s1);
     float *invd = reinterpret_cast<float *>(base + kStoredInvDOff);
     for (int l = threadIdx.x; l < kK; l += blockDim.x) {
@@ -1990,7 +2321,7 @@ __global__ void __launch_bounds__(512) build_c_scales_kernel(const double *g64, 
 int build_stored_c(rljsde_plan *p, const double *d_g64)
 {
     if (!p->d_cstore || p->n_stored < 1 || p->n_stored > 65535) return RLJSDE_ERR_INVALID_ARG;
-    build_c_kernel<<<dim3(kK, p->n_stored), 512>>>(d_g64, p->d_consts, p->slot_ap,
+    build_c_kernel<<<dim3(kK, p->n_stored), 512>>>(d_g64, p->d_consts, p->slot_ap, p->params.pairs,
                                                   static_cast<float4 *>(p->d_cstore));
     build_c_scales_kernel<<<p->n_stored, 512>>>(d_g64, static_cast<float4 *>(p->d_cstore));
     if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) return RLJSDE_ERR_CUDA;
@@ -2031,22 +2362,8 @@ int choose_launch(rljsde_plan *p, int warps, int ctas_per_sm)
     const int fp64 = p->params.precision == 1;
     const int mode = (p->kind == 1 ? 3 : p->kind == 3 ? 4 : 0) | (p->params.pairs ? kModePairs : 0);
     if (p->n_stored > 0 && !fp64) {
-        // the stored-C loop: 8 warps in one CTA per SM, or 4 warps x 3 CTAs for
-        // short loops where that instantiation exists
-        const int want_warps = p->params.nu_max >= 20 ? 8 : 4;
-        p->variant_stored = -1;
-        for (int i = 0; i < kNumVariants; ++i)
-            if (!kVariants[i].fp64 && kVariants[i].mode == (mode | kModeStoredC) &&
-                (p->variant_stored < 0 || kVariants[i].warps == want_warps))
-                p->variant_stored = i;
-        if (p->variant_stored < 0) return RLJSDE_ERR_UNSUPPORTED;
-        const int occ = occupancy(kVariants[p->variant_stored]);
-        if (occ < 0) return RLJSDE_ERR_CUDA;
-        if (occ == 0) return RLJSDE_ERR_UNSUPPORTED;
-        long long g = (long long)p->sm_count * occ;
-        p->grid_stored = (int)(p->n_chunks < g ? (p->n_chunks > 0 ? p->n_chunks : 1) : g);
-        p->ctas_stored = occ;
-        p->warps_stored = kVariants[p->variant_stored].warps;
+        stored_shape(p, stored_kind(p), p->warps_stored, p->grid_stored);       // for rljsde_plan_info
+        p->ctas_stored = 1;
     }
     // The variant with this precision and warp count whose register budget
     // admits the requested CTAs per SM (the largest one not above it).
@@ -2121,7 +2438,11 @@ int rljsde_reconstruct_learned(const rljsde_plan_t *plan, const float *lr, size_
     const int sc = plan->n_stored > 0 && plan->n_stored == plan->n_tables ? kModeStoredC : 0;
     const int lw = sc ? 4 : plan->learned_warps, lm = sc ? 3 : plan->learned_minb;
     int st = launch_mode(plan, a, 1 | sc, lw, lm, (cudaStream_t)stream);
-    if (st == RLJSDE_OK) st = launch_mode(plan, a, 2 | sc, 4, 0, (cudaStream_t)stream);
+    if (st == RLJSDE_OK && sc) {
+        st = launch_stored(plan, a, kFallback, (cudaStream_t)stream);
+    } else if (st == RLJSDE_OK) {
+        st = launch_mode(plan, a, 2, 4, 0, (cudaStream_t)stream);
+    }
     return st;
 }
 

@@ -234,6 +234,7 @@ void release(rljsde_plan *p)
     cudaFree(p->d_records_short);
     cudaFree(p->d_cstore);
     cudaFree(p->d_cslot);
+    cudaFree(p->d_order);
     cudaFree(p->d_entries);
     cudaFree(p->d_chunk_table);
     cudaFree(p->d_consts);
@@ -555,6 +556,19 @@ int create(rljsde_plan **out, int n_images, const uint8_t *const *masks, const i
                 }
                 if (!st) st = upload(&d_g64, g64.data(), g64.size() * sizeof(double));
                 if (!st) st = upload(&p->d_cslot, p->cslot.data(), p->cslot.size() * sizeof(int));
+                if (!st) {
+                    std::vector<uint32_t> order;
+                    order.reserve((size_t)p->n_stored_blocks);
+                    for (int e = 0; e < p->n_entries; ++e)
+                        if (entries[e].img >= 0 && p->cslot[chunk_table[e / kChunk]] >= 0) order.push_back((uint32_t)e);
+                    p->n_order = (int)order.size();
+                    // D and h_t are mirror-exact (D_k = D_-k bit for bit), so the scaled
+                    // columns are too whenever the frequency weight is
+                    p->mirror = 1;
+                    for (int k = 0; k < kK; ++k)
+                        if (p->q[k] != p->q[((32 - k / kW) & 31) * kW + ((32 - k % kW) & 31)]) p->mirror = 0;
+                    st = upload(&p->d_order, order.data(), order.size() * sizeof(uint32_t));
+                }
                 if (!st) st = build_stored_c(p, d_g64);
                 cudaFree(d_g64);
             }

@@ -114,10 +114,10 @@ static_assert(sizeof(Shortlist) == 136, "shortlist layout");
 // state being R'_k = s_k R_k with s_k = sqrt(q_k / D_k), so that the score
 // of Eq. 11 is |R'_k|^2:
 //   C'_{k,l} = s_k C_{k,l}: 1024 columns of 8 KiB, each as 16 x 32 float4
-//     (C'_{k,l}.re, C'_{k+32,l}.re, C'_{k,l}.im, C'_{k+32,l}.im), entry
-//     i * 32 + lane holding the two candidates that lane of the FP32 loop
-//     updates in its register pair i;
-//   then s_k in the same lane order, as float4 (s_k, s_k+32, s_k, s_k+32);
+//     (C'_{k,l}.re, C'_{k',l}.re, C'_{k,l}.im, C'_{k',l}.im), entry i * 32 +
+//     lane holding the two candidates k, k' that lane of the stored-C loop
+//     updates in its register pair i (slot_k, pair_slot in kernels.cu);
+//   then s_k in the same lane order, as float4 (s_k, s_k', s_k, s_k');
 //   then 1 / (s_l D_l) by linear l (0 where s_l D_l is 0), so that
 //     delta = R_uv / D_uv = R'_uv / (s_uv D_uv) (Eq. 16).
 constexpr size_t kStoredColsBytes = (size_t)kK * kK * 8;
@@ -148,7 +148,7 @@ struct rljsde_plan {
     int n_apertures = 0;              // distinct non-empty apertures in the masks
     int device = 0, sm_count = 0;
     int warps = 4, ctas_per_sm = 0, grid = 0, variant = 0;   // factored loop (and FP64, learned)
-    int variant_stored = 0, grid_stored = 0, ctas_stored = 0, warps_stored = 0;   // stored-C loop, if n_stored > 0
+    int grid_stored = 0, ctas_stored = 0, warps_stored = 0;   // stored-C loop, if n_stored > 0
     int learned_warps = 4;            // warps per CTA of the shortlist-loop kernel (4: two blocks per warp)
     int learned_minb = 3;             // its register budget: resident CTAs per SM
     // device memory, all owned by the plan
@@ -159,6 +159,9 @@ struct rljsde_plan {
     int n_stored_blocks = 0;          // blocks that use them
     std::vector<int> cslot;           // per table set: its stored matrix, or -1 (factored)
     int *d_cslot = nullptr;
+    uint32_t *d_order = nullptr;      // entries of the stored table sets, in work-list order without padding
+    int n_order = 0;
+    int mirror = 0;                   // q_k = q_-k: column -l is the conjugate mirror of column l
     void *d_cstore = nullptr;         // n_stored x kStoredTableBytes, in the stored-C loop's read order
     size_t cstore_bytes = 0;
     rljsde::WorkEntry *d_entries = nullptr;
