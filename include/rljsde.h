@@ -113,10 +113,13 @@ typedef struct {
                              memory, one more kernel); 0 = auto (default):
                              stored for every table set, the most used first,
                              while the matrices fit in an eighth of the free
-                             device memory, factored for the rest and for FP64
-                             loops, paths 2 and 3 and frequency weights with a
-                             zero (the stored loop's state is sqrt(q / D) R,
-                             which cannot hold R where q is 0).  1 and 3 need
+                             device memory, factored for the rest, for paths 2
+                             and 3 and for frequency weights with a zero (the
+                             FP32 stored loop's state is sqrt(q / D) R, which
+                             cannot hold R where q is 0).  FP64 plans store
+                             FP64 matrices (16 MiB per table set) by the same
+                             rule where a single reconstruction earns their
+                             build back, except with pairs.  1 and 3 need
                              the FP32 loop on path 1 and q > 0 wherever it
                              counts (RLJSDE_ERR_UNSUPPORTED otherwise, also
                              when auto would choose path 2 or 3) and fail with

@@ -138,6 +138,7 @@ struct Args {
     const int *cslot;                      // per table set: its stored matrix, or -1 (factored)
     int cfilter;                           // chunks a factored launch takes: 0 all, 1 those whose table
                                            // set has no stored matrix
+    const unsigned char *cstore64;         // the same for FP64 plans, kStored64Bytes each
     const uint32_t *order;                 // stored-C loop: the entries of the stored table sets
     int n_order;
     const Consts *consts;
@@ -462,6 +463,46 @@ __device__ __forceinline__ void select_step(const Args &a, const C2<T> *om, cons
     }
 }
 
+// R at the four candidates (k1 + 16 a, k2 + 16 b), entry 2 a + b, of one
+// frequency group from its factored state.
+template <typename T, int LAY>
+__device__ __forceinline__ void group_to_R(const Args &a, const C2<T> (&Yi)[4], const C2<T> e1, const C2<T> *omc,
+                                           const int k1, const int k2, C2<T> (&R)[4])
+{
+                // R_k = sum_s conj(e_s(k)) Z_s, e = (1, w^k2, w^k1, w^(k1+k2)), with Z_s the
+                // sum of Y_t over the slots t whose aperture holds sub-pixel s
+                // (three-quarter: Z_s = S - Y_s, S = sum_t Y_t; single: Z_s = Y_s)
+                C2<T> Z[4];
+                if constexpr (LAY == kLaySingle) {
+    #pragma unroll
+                    for (int sp = 0; sp < 4; ++sp) Z[sp] = Yi[sp];
+                } else if constexpr (LAY == kLayGeneral) {
+    #pragma unroll
+                    for (int sp = 0; sp < 4; ++sp) {
+                        Z[sp] = {0, 0};
+    #pragma unroll
+                        for (int t = 0; t < 4; ++t)
+                            if ((a.slot_ap >> (4 * t + sp)) & 1u) Z[sp] = cadd(Z[sp], Yi[t]);
+                    }
+                } else {
+                    // Z_s = S - Y_s as the sum of the other three: 6 additions, no cancellation
+                    const C2<T> P01 = cadd(Yi[0], Yi[1]), P23 = cadd(Yi[2], Yi[3]);
+                    Z[0] = cadd(Yi[1], P23);
+                    Z[1] = cadd(Yi[0], P23);
+                    Z[2] = cadd(P01, Yi[3]);
+                    Z[3] = cadd(P01, Yi[2]);
+                }
+                const C2<T> Z0 = Z[0];
+                const C2<T> U = cmul(e1, Z[1]);
+                const C2<T> V = cmul(omc[k1], Z[2]);
+                const C2<T> X = cmul(omc[(k1 + k2) & 31], Z[3]);
+                const C2<T> pp = cadd(Z0, U), mm = csub(Z0, U), ss = cadd(V, X), dd = csub(V, X);
+                R[0] = cadd(pp, ss);
+    R[1] = cadd(mm, dd);
+    R[2] = csub(pp, ss);
+    R[3] = csub(mm, dd);
+}
+
 // ------------------------------------------------------ FP64 (scalar) loop --
 template <typename T, int LAY = kLayThreeQuarter, bool PAIRS = false>
 __device__ __forceinline__ void greedy_loop(const Args &a, const Record<T> &rec, const C2<T> *om,
@@ -502,35 +543,9 @@ __device__ __forceinline__ void greedy_loop(const Args &a, const Record<T> &rec,
                     Y[i][3] = csub(Y[i][3], cmul(C2<T>{pw * g[3].re, -pw * g[3].im}, C2<T>{H23.z, H23.w}));
                 }
             }
-            // R_k = sum_s conj(e_s(k)) Z_s, e = (1, w^k2, w^k1, w^(k1+k2)), with Z_s the
-            // sum of Y_t over the slots t whose aperture holds sub-pixel s
-            // (three-quarter: Z_s = S - Y_s, S = sum_t Y_t; single: Z_s = Y_s)
-            C2<T> Z[4];
-            if constexpr (LAY == kLaySingle) {
-#pragma unroll
-                for (int sp = 0; sp < 4; ++sp) Z[sp] = Y[i][sp];
-            } else if constexpr (LAY == kLayGeneral) {
-#pragma unroll
-                for (int sp = 0; sp < 4; ++sp) {
-                    Z[sp] = {0, 0};
-#pragma unroll
-                    for (int t = 0; t < 4; ++t)
-                        if ((a.slot_ap >> (4 * t + sp)) & 1u) Z[sp] = cadd(Z[sp], Y[i][t]);
-                }
-            } else {
-                // Z_s = S - Y_s as the sum of the other three: 6 additions, no cancellation
-                const C2<T> P01 = cadd(Y[i][0], Y[i][1]), P23 = cadd(Y[i][2], Y[i][3]);
-                Z[0] = cadd(Y[i][1], P23);
-                Z[1] = cadd(Y[i][0], P23);
-                Z[2] = cadd(P01, Y[i][3]);
-                Z[3] = cadd(P01, Y[i][2]);
-            }
-            const C2<T> Z0 = Z[0];
-            const C2<T> U = cmul(e1, Z[1]);
-            const C2<T> V = cmul(omc[k1], Z[2]);
-            const C2<T> X = cmul(omc[(k1 + k2) & 31], Z[3]);
-            const C2<T> pp = cadd(Z0, U), mm = csub(Z0, U), ss = cadd(V, X), dd = csub(V, X);
-            const C2<T> R00 = cadd(pp, ss), R01 = cadd(mm, dd), R10 = csub(pp, ss), R11 = csub(mm, dd);
+            C2<T> R4[4];
+            group_to_R<T, LAY>(a, Y[i], e1, omc, k1, k2, R4);
+            const C2<T> R00 = R4[0], R01 = R4[1], R10 = R4[2], R11 = R4[3];
             const Vec4<T> qd = ld4(&rec.qD[k1 * 16 + k2]);
             const int k = k1 * kW + k2;
             keep_best(key32(qd.x * (R00.re * R00.re + R00.im * R00.im)), k, R00.re, R00.im, bs0, bk0, b0re, b0im);
@@ -782,6 +797,7 @@ __host__ __device__ constexpr int slot_pair(int s)
 __host__ __device__ constexpr int slot_half(int s) { return pair_slot(slot_pair(s), 1) == s; }
 // lane that holds candidate k
 __host__ __device__ constexpr int lane_of(int k) { return (k >> 5) <= 16 ? (k & 31) : ((32 - (k & 31)) & 31); }
+__host__ __device__ constexpr int mirror_of(int k) { return (((32 - (k >> 5)) & 31) << 5) | ((32 - k) & 31); }   // -k
 // candidate of a lane's slot
 __host__ __device__ constexpr int slot_k(int s, int lane) { return s * kW + (s <= 16 ? lane : ((32 - lane) & 31)); }
 
@@ -1036,7 +1052,7 @@ __device__ __forceinline__ void stored_block(const Args &a, const float4 *cs, co
         const int bk = stored_argmax(R, lane);
         const bool more = it + 1 < a.nu_max;
         // column uv, or -uv to be read conjugated with the pairs' places exchanged
-        const int mk = (((32 - (bk >> 5)) & 31) << 5) | ((32 - bk) & 31);       // -uv
+        const int mk = mirror_of(bk);
         const bool mir = MIRROR && mk < bk;
         float4 col[16];
         if (more) {
@@ -1722,7 +1738,7 @@ __device__ __forceinline__ void fill_tables(const Args &a, C2<float> *om, C2<flo
     }
 }
 
-enum StoredKind { kSolo, kSoloMirror, kSoloPairs, kFallback };
+enum StoredKind { kSolo, kSoloMirror, kSoloPairs, kFallback, kFp64 };
 // Warps per CTA (one CTA per SM).  Twelve is three per scheduler at 168
 // registers: the loop is bound by the latency of its own instructions (issue
 // active 52 %, ALU and FMA pipes 42 %, no memory unit above 58 %), and the
@@ -1730,7 +1746,7 @@ enum StoredKind { kSolo, kSoloMirror, kSoloPairs, kFallback };
 // 100: 2.82 against 3.24 ms); sixteen at 128 registers spill (8.3 ms, 3.4 ms
 // with the column loaded in two halves).  The mirrored loop runs where blocks
 // are few and keeps eight and no spills (64x64: 60 against 64 us).
-constexpr int stored_warps(const int kind) { return kind == kSoloMirror ? 8 : kStoredWarps; }
+constexpr int stored_warps(const int kind) { return kind == kSoloMirror || kind == kFp64 ? 8 : kStoredWarps; }
 
 template <int LAY, int KIND, bool TRACE>
 __global__ void __launch_bounds__(stored_warps(KIND) * 32, 1) stored_kernel(const Args a)
@@ -1784,6 +1800,151 @@ __global__ void __launch_bounds__(stored_warps(KIND) * 32, 1) stored_kernel(cons
                 if (i >= n_list) break;
                 block(list[i]);
             }
+        }
+    }
+}
+
+// ------------------------------------------------ stored-C FP64 kernel --
+// The FP64 loop with the Gram matrices stored in FP64 (16 MiB per table set):
+// the state is R itself and Eq. 17 is one complex multiply-add per candidate,
+// 4 FP64 instructions, where the factored loop rebuilds R from four type
+// planes (about 18).  GB300 executes two FP64 lanes per SM and cycle, 1/64 of
+// the FP32 rate, so nothing else matters: the scores are screened in FP32 from
+// the top bits of R (integer operations; an FP64-to-FP32 conversion would cost
+// as much as a multiply-add) and only candidates within 2^-18 of the largest
+// screened score get their FP64 score, rounded to binary32 as before.  The
+// screen's relative error is below 2^-20: R's components are truncated to 24
+// bits (2^-23), q / D and the four operations round at 2^-24 each.
+//
+// Lane (kap2 = lane & 15, h = lane >> 4) holds slots s = 16 a + 2 i + b, k =
+// (8 h + i + 16 a, kap2 + 16 b): increasing k, the initial projection's layout.
+// Table set: 1024 columns of [slot][lane] (re, im); q / D then 1 / D by k in
+// FP64; q / D rounded to FP32 as [slot][lane].
+// 256x256, nu_max 100: 21.3 -> 3.6 ms, 151 FP64 instructions an iteration (FP64 floor 2.0 ms).
+__host__ __device__ constexpr int slot64_k(int s, int lane)
+{
+    return (8 * (lane >> 4) + ((s >> 1) & 7) + 16 * (s >> 4)) * kW + (lane & 15) + 16 * (s & 1);
+}
+__host__ __device__ constexpr int slot64_of(int k) { return 16 * (k >> 9) + 2 * ((k >> 5) & 7) + ((k >> 4) & 1); }
+__host__ __device__ constexpr int lane64_of(int k) { return 16 * ((k >> 8) & 1) + (k & 15); }
+constexpr int kStored64Warps = 8;
+struct Stored64Smem {
+    static constexpr size_t off_scratch = 0;                                     // kStored64Warps x 8 KB
+    static constexpr size_t off_om = kStored64Warps * 256 * 2 * sizeof(C2<double>);
+    static constexpr size_t off_omc = off_om + 32 * sizeof(C2<double>);
+    static constexpr size_t off_w = off_omc + 32 * sizeof(C2<double>);
+    static constexpr size_t bytes = off_w + 256 * sizeof(double);
+};
+
+// |x| truncated to 24 significant bits as a float (0 below 2^-127; the
+// caller looks at `top`, the largest biased-down exponent word, for values a
+// float does not hold).
+__device__ __forceinline__ float screen(const double x, int &top)
+{
+    const int e = max((__double2hiint(x) & 0x7fffffff) - (896 << 20), 0);
+    top = max(top, e);
+    return __uint_as_float(__funnelshift_l((unsigned)__double2loint(x), (unsigned)e, 3));
+}
+
+template <int LAY>
+__global__ void __launch_bounds__(kStored64Warps * 32, 1) stored64_kernel(const Args a)
+{
+    using L = Stored64Smem;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    C2<double> *scratch = reinterpret_cast<C2<double> *>(smem + L::off_scratch) + warp * 512;
+    C2<double> *om = reinterpret_cast<C2<double> *>(smem + L::off_om);
+    C2<double> *omc = reinterpret_cast<C2<double> *>(smem + L::off_omc);
+    double *wt = reinterpret_cast<double *>(smem + L::off_w);
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) wt[i] = a.consts->w64[i];
+    for (int i = threadIdx.x; i < 32; i += blockDim.x) {
+        om[i] = {a.consts->om64[2 * i], a.consts->om64[2 * i + 1]};
+        omc[i] = {a.consts->om64[2 * i], -a.consts->om64[2 * i + 1]};
+    }
+    __syncthreads();
+    const int k2 = lane & 15, h = lane >> 4;
+    const int eta = kOff + ((lane >> 2) & 3), gam = kOff + (lane & 3);
+    for (int o = blockIdx.x * warps + warp; o < a.n_order; o += gridDim.x * warps) {
+        const uint32_t e = a.order[o];
+        const WorkEntry we = a.entries[e];
+        const uint32_t t = a.chunk_table[e / kChunk];
+        const unsigned char *tab = a.cstore64 + (size_t)a.cslot[t] * kStored64Bytes;
+        const double *qd = reinterpret_cast<const double *>(tab + kStored64ColsBytes), *invd = qd + kK;
+        const float *qf = reinterpret_cast<const float *>(invd + kK) + lane;
+        C2<double> R[32];
+        {
+            const uint8_t *types = a.records + (size_t)t * sizeof(Record<double>) + offsetof(Record<double>, types);
+            C2<double> Y[8][4];
+            initial_projection<double>(a, types, scratch, omc, wt, we, lane, Y);
+            const C2<double> e1 = omc[k2];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                C2<double> r4[4];
+                group_to_R<double, LAY>(a, Y[i], e1, omc, 8 * h + i, k2, r4);
+                R[2 * i] = r4[0]; R[2 * i + 1] = r4[1]; R[16 + 2 * i] = r4[2]; R[16 + 2 * i + 1] = r4[3];
+            }
+        }
+        double fpix = 0;
+        const long long trow = (long long)we.ord * a.nu_max;
+        for (int it = 0;;) {
+            float s32[32], m = 0.f;
+            int top = 0;
+#pragma unroll
+            for (int s = 0; s < 32; ++s) {
+                const float re = screen(R[s].re, top), im = screen(R[s].im, top);
+                s32[s] = ldg_stream1(qf + 32 * s) * fmaf(re, re, im * im);
+                m = fmaxf(m, s32[s]);
+            }
+            const float M = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));
+            // outside the floats' safe range every candidate gets its FP64 score
+            const bool every = __any_sync(0xffffffffu, top >= ((127 + 60) << 20)) || !(M >= 0x1p-100f && M <= 0x1p+100f);
+            const float least = every ? -1.f : M * (1.f - 0x1p-18f);
+            // slots any lane has to look at: a branch over each of the others
+            // (predicated, their FP64 instructions would still take the pipe)
+            unsigned hits = 0;
+#pragma unroll
+            for (int s = 0; s < 32; ++s)
+                if (every || s32[s] >= least) hits |= 1u << s;
+            const unsigned any = __reduce_or_sync(0xffffffffu, hits);
+            unsigned bits = 0;                            // binary32 score + 1, 0 = none
+            int bk = kK - 1;
+            double bre = 0, bim = 0;
+#pragma unroll
+            for (int s = 0; s < 32; ++s)
+                if ((any >> s) & 1u) {
+                    asm volatile("" ::: "memory");
+                    const int k = slot64_k(s, lane);
+                    const float key = (float)(qd[k] * (R[s].re * R[s].re + R[s].im * R[s].im));
+                    if (((hits >> s) & 1u) && __float_as_uint(key) + 1 > bits) {
+                        bits = __float_as_uint(key) + 1; bk = k; bre = R[s].re; bim = R[s].im;
+                    }
+                }
+            const unsigned most = __reduce_max_sync(0xffffffffu, bits);
+            bk = (int)__reduce_min_sync(0xffffffffu, bits == most ? (unsigned)bk : (unsigned)(kK - 1));
+            const int wl = (bk & 15) + ((bk >> 5) & 8) * 2;
+            const double Rre = __shfl_sync(0xffffffffu, bre, wl), Rim = __shfl_sync(0xffffffffu, bim, wl);
+            const double invD = invd[bk];
+            const C2<double> gd = {a.gamma * (Rre * invD), a.gamma * (Rim * invD)};   // gamma delta (Eqs. 15, 16)
+            const C2<double> ph = om[(eta * (bk >> 5) + gam * (bk & 31)) & 31];
+            fpix += gd.re * ph.re - gd.im * ph.im;
+            if (a.trace_sel != nullptr && lane == 0) {
+                a.trace_sel[trow + it] = (uint16_t)bk;
+                a.trace_dc[2 * (trow + it)] = (float)gd.re;
+                a.trace_dc[2 * (trow + it) + 1] = (float)gd.im;
+            }
+            if (++it >= a.nu_max) break;
+            const double2 *col = reinterpret_cast<const double2 *>(tab) + (size_t)bk * kK + lane;
+#pragma unroll
+            for (int s = 0; s < 32; ++s) {
+                const double2 c = __ldg(col + 32 * s);
+                R[s].re = fma(gd.im, c.y, fma(-gd.re, c.x, R[s].re));
+                R[s].im = fma(-gd.im, c.x, fma(-gd.re, c.y, R[s].im));
+            }
+        }
+        if (lane < 16) {
+            const ImageDesc img = a.descs ? a.descs[we.img] : a.single;
+            const int yy = 4 * we.bi + (lane >> 2), xx = 4 * we.bj + (lane & 3);
+            img.hr[(long long)yy * img.hr_pitch + xx] = (float)fpix;
         }
     }
 }
@@ -2127,6 +2288,7 @@ Args make_args(const rljsde_plan *p)
     a.records = static_cast<const unsigned char *>(p->d_records);
     a.records_short = static_cast<const unsigned char *>(p->d_records_short);
     a.cstore = static_cast<const float4 *>(p->d_cstore);
+    a.cstore64 = static_cast<const unsigned char *>(p->d_cstore);
     a.cslot = p->d_cslot;
     a.order = p->d_order;
     a.n_order = p->n_order;
@@ -2174,6 +2336,7 @@ StoredFn stored_fn(const rljsde_plan *p, const int kind, const bool trace)
 constexpr int kMirrorBlocksPerSm = 27;
 int stored_kind(const rljsde_plan *p)
 {
+    if (p->params.precision == 1) return kFp64;
     if (p->params.pairs) return kSoloPairs;
     return p->mirror && p->n_order <= kMirrorBlocksPerSm * p->sm_count ? kSoloMirror : kSolo;
 }
@@ -2201,6 +2364,16 @@ int launch_stored(const rljsde_plan *p, const Args &a, const int kind, cudaStrea
     return cudaGetLastError() == cudaSuccess ? RLJSDE_OK : RLJSDE_ERR_CUDA;
 }
 
+int launch_stored64(const rljsde_plan *p, const Args &a, cudaStream_t s)
+{
+    const StoredFn fn = p->kind == 1 ? stored64_kernel<kLayGeneral>
+                        : p->kind == 3 ? stored64_kernel<kLaySingle> : stored64_kernel<kLayThreeQuarter>;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Stored64Smem::bytes) != cudaSuccess)
+        return RLJSDE_ERR_CUDA;
+    fn<<<p->grid_stored, p->warps_stored * 32, Stored64Smem::bytes, s>>>(a);
+    return cudaGetLastError() == cudaSuccess ? RLJSDE_OK : RLJSDE_ERR_CUDA;
+}
+
 int launch(const rljsde_plan *p, const Args &a, cudaStream_t s)
 {
     if (p->direct) {
@@ -2213,7 +2386,7 @@ int launch(const rljsde_plan *p, const Args &a, cudaStream_t s)
         // factored loop on the others: one launch each (one kernel holding
         // both loops spills and ran the stored loop 1.5x slower)
         if (p->n_stored > 0) {
-            const int st = launch_stored(p, a, stored_kind(p), s);
+            const int st = p->params.precision == 1 ? launch_stored64(p, a, s) : launch_stored(p, a, stored_kind(p), s);
             if (st != RLJSDE_OK) return st;
         }
         if (p->n_stored < p->n_tables) {
@@ -2247,8 +2420,7 @@ int launch_mode(const rljsde_plan *p, const Args &a, int mode, int warps, int mi
 // scaled by s_k = sqrt(q_k / D_k) (the stored-C loop's state is s R),
 // evaluated in FP64 from the FP64 tables and rounded to FP32 once, in the
 // loop's read order (float4 i * 32 + lane of column l: the candidates of
-// lane's register pair i).  One CTA per (column, stored table set), one
-// thread per float4.
+// lane's register pair i).
 __device__ __forceinline__ C2<double> h64(const double2 *om, const uint32_t slot_ap, const int t, const int k1,
                                           const int k2)
 {
@@ -2264,38 +2436,91 @@ __device__ __forceinline__ C2<double> h64(const double2 *om, const uint32_t slot
     return z;
 }
 
+// One CTA per kBuildCols columns and stored table set, one thread per float4
+// (two candidates); h_t(k) of its candidates stays in a thread's registers,
+// h_t(l) in shared memory.  Only the columns l <= -l are evaluated: column -l
+// is C_{-k,-l} = conj(C_{k,l}), bit for bit (the tables are mirror-exact).
+// The same operations per entry as evaluating everything on the spot, a sixth
+// of the FP64 work, which bounds it.
+// With FP64 the entries are stored unscaled in FP64, for stored64_kernel.
+constexpr int kBuildCols = 16;
+constexpr int kCanonical = 514;                    // columns l with l <= -l: (0, 0..16), rows 1..15, (16, 0..16)
+__host__ __device__ constexpr int canonical_column(int c) { return c < 17 ? c : c + 15; }
+template <bool FP64>
 __global__ void __launch_bounds__(512) build_c_kernel(const double *g64, const Consts *consts,
-                                                      const uint32_t slot_ap, const int pairs, float4 *out)
+                                                      const uint32_t slot_ap, const int pairs, unsigned char *out)
 {
     __shared__ double2 G[4][256];
     __shared__ double2 om[32];
-    const int l = blockIdx.x, tab = blockIdx.y;
+    __shared__ C2<double> hl[kBuildCols][4];
+    const int c0 = blockIdx.x * kBuildCols, tab = blockIdx.y;
     const double *src = g64 + (size_t)tab * kStoredBuildDoubles;
     for (int i = threadIdx.x; i < 1024; i += blockDim.x) G[i >> 8][i & 255] = make_double2(src[2 * i], src[2 * i + 1]);
     if (threadIdx.x < 32) om[threadIdx.x] = make_double2(consts->om64[2 * threadIdx.x], consts->om64[2 * threadIdx.x + 1]);
     __syncthreads();
-    const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int l1 = l >> 5, l2 = l & 31;
-    float re[2], im[2];
-    for (int e = 0; e < 2; ++e) {
-        const int k = slot_k(pair_slot(i, e), lane), k1 = k >> 5, k2 = k & 31;
-        const int d = ((l1 - k1) & 15) * 16 + ((l2 - k2) & 15);
-        double cre = 0.0, cim = 0.0;
-        for (int t = 0; t < 4; ++t) {
-            const C2<double> hk = h64(om, slot_ap, t, k1, k2), hl = h64(om, slot_ap, t, l1, l2);
-            const C2<double> z = cmul(cconj(hk), hl);
-            const double2 gt = G[t][d];
-            cre += z.re * gt.x - z.im * gt.y;
-            cim += z.re * gt.y + z.im * gt.x;
-        }
-        // conjugate-pair plans: the rows of the hidden member -k carry k's scale
-        const int mk = ((32 - k1) & 31) * kW + ((32 - k2) & 31);
-        const double sk = sqrt(src[2048 + (pairs && mk < k ? mk : k)]);
-        re[e] = (float)(sk * cre);
-        im[e] = (float)(sk * cim);
+    if (threadIdx.x < kBuildCols * 4) {
+        const int l = canonical_column(min(c0 + (int)threadIdx.x / 4, kCanonical - 1)), t = threadIdx.x & 3;
+        hl[threadIdx.x / 4][t] = h64(om, slot_ap, t, l >> 5, l & 31);
     }
-    out[(size_t)tab * (kStoredTableBytes / 16) + (size_t)l * 512 + threadIdx.x] =
-        make_float4(re[0], re[1], im[0], im[1]);
+    const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int k[2];
+    C2<double> hk[2][4];
+    double sk[2], sm[2];                           // row scales of k and -k
+    for (int e = 0; e < 2; ++e) {
+        k[e] = FP64 ? slot64_k(2 * i + e, lane) : slot_k(pair_slot(i, e), lane);
+        for (int t = 0; t < 4; ++t) hk[e][t] = cconj(h64(om, slot_ap, t, k[e] >> 5, k[e] & 31));
+        // conjugate-pair plans: the rows of the hidden member -k carry k's scale
+        const int mk = mirror_of(k[e]);
+        sk[e] = FP64 ? 1.0 : sqrt(src[2048 + (pairs && mk < k[e] ? mk : k[e])]);
+        sm[e] = FP64 ? 1.0 : sqrt(src[2048 + (pairs && k[e] < mk ? k[e] : mk)]);
+    }
+    __syncthreads();
+    for (int c = 0; c < kBuildCols && c0 + c < kCanonical; ++c) {
+        const int l = canonical_column(c0 + c), l1 = l >> 5, l2 = l & 31, ml = mirror_of(l);
+        double2 v[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int d = ((l1 - (k[e] >> 5)) & 15) * 16 + ((l2 - k[e]) & 15);
+            double cre = 0.0, cim = 0.0;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const C2<double> z = cmul(hk[e][t], hl[c][t]);
+                const double2 gt = G[t][d];
+                cre += z.re * gt.x - z.im * gt.y;
+                cim += z.re * gt.y + z.im * gt.x;
+            }
+            v[e] = make_double2(cre, cim);
+        }
+        if constexpr (FP64) {
+            double2 *o = reinterpret_cast<double2 *>(out + (size_t)tab * kStored64Bytes);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                o[(size_t)l * kK + (2 * i + e) * 32 + lane] = v[e];
+                const int m = mirror_of(k[e]);
+                if (ml != l) o[(size_t)ml * kK + slot64_of(m) * 32 + lane64_of(m)] = make_double2(v[e].x, -v[e].y);
+            }
+        } else {
+            float4 *o = reinterpret_cast<float4 *>(out + (size_t)tab * kStoredTableBytes);
+            o[(size_t)l * 512 + threadIdx.x] = make_float4((float)(sk[0] * v[0].x), (float)(sk[1] * v[1].x),
+                                                           (float)(sk[0] * v[0].y), (float)(sk[1] * v[1].y));
+            // the mirrors of register pair i: pair i ^ 8 of the lane, but pair 0 in lane -L and pair 8 with its halves exchanged
+            const float4 m = make_float4((float)(sm[0] * v[0].x), (float)(sm[1] * v[1].x), (float)(sm[0] * -v[0].y),
+                                         (float)(sm[1] * -v[1].y));
+            if (ml != l)
+                o[(size_t)ml * 512 + (i == 0 ? (32 - lane) & 31 : i == 8 ? 256 + lane : (i ^ 8) * 32 + lane)] =
+                    i == 8 ? make_float4(m.y, m.x, m.w, m.z) : m;
+        }
+    }
+}
+
+// q / D and 1 / D of an FP64 table set (see stored64_kernel).
+__global__ void __launch_bounds__(512) build_c64_tables_kernel(const double *g64, unsigned char *out)
+{
+    const double *src = g64 + (size_t)blockIdx.x * kStoredBuildDoubles + 2048;
+    double *d = reinterpret_cast<double *>(out + (size_t)blockIdx.x * kStored64Bytes + kStored64ColsBytes);
+    float *qf = reinterpret_cast<float *>(d + 2 * kK);
+    for (int i = threadIdx.x; i < 2 * kK; i += blockDim.x) d[i] = src[i];
+    for (int i = threadIdx.x; i < kK; i += blockDim.x) qf[i] = (float)src[slot64_k(i >> 5, i & 31)];
 }
 
 // The row scales s_k in the lane order and 1 / (s_l D_l) of each stored
@@ -2321,9 +2546,15 @@ __global__ void __launch_bounds__(512) build_c_scales_kernel(const double *g64, 
 int build_stored_c(rljsde_plan *p, const double *d_g64)
 {
     if (!p->d_cstore || p->n_stored < 1 || p->n_stored > 65535) return RLJSDE_ERR_INVALID_ARG;
-    build_c_kernel<<<dim3(kK, p->n_stored), 512>>>(d_g64, p->d_consts, p->slot_ap, p->params.pairs,
-                                                  static_cast<float4 *>(p->d_cstore));
-    build_c_scales_kernel<<<p->n_stored, 512>>>(d_g64, static_cast<float4 *>(p->d_cstore));
+    const dim3 grid((kCanonical + kBuildCols - 1) / kBuildCols, p->n_stored);
+    unsigned char *out = static_cast<unsigned char *>(p->d_cstore);
+    if (p->params.precision == 1) {
+        build_c_kernel<true><<<grid, 512>>>(d_g64, p->d_consts, p->slot_ap, p->params.pairs, out);
+        build_c64_tables_kernel<<<p->n_stored, 512>>>(d_g64, out);
+    } else {
+        build_c_kernel<false><<<grid, 512>>>(d_g64, p->d_consts, p->slot_ap, p->params.pairs, out);
+        build_c_scales_kernel<<<p->n_stored, 512>>>(d_g64, static_cast<float4 *>(p->d_cstore));
+    }
     if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) return RLJSDE_ERR_CUDA;
     return RLJSDE_OK;
 }
@@ -2361,7 +2592,7 @@ int choose_launch(rljsde_plan *p, int warps, int ctas_per_sm)
     if (warps == 0) { warps = 4; if (ctas_per_sm == 0) ctas_per_sm = 3; }
     const int fp64 = p->params.precision == 1;
     const int mode = (p->kind == 1 ? 3 : p->kind == 3 ? 4 : 0) | (p->params.pairs ? kModePairs : 0);
-    if (p->n_stored > 0 && !fp64) {
+    if (p->n_stored > 0) {
         stored_shape(p, stored_kind(p), p->warps_stored, p->grid_stored);       // for rljsde_plan_info
         p->ctas_stored = 1;
     }

@@ -147,11 +147,26 @@ inline double inv_or_zero(double num, double den) { return den > 1e-300 ? num / 
 // other member of each pair gets q/D = 0.
 inline bool pair_hidden(bool pairs, int k) { return pairs && ((-(k / kW)) & 31) * kW + ((-(k % kW)) & 31) < k; }
 
+// FP64 tables for the stored Gram matrix: G_t [t][d] as (re, im), q/D, 1/D.
+void build_tables64(const Tables &T, bool pairs, const std::vector<double> &q, double *g64)
+{
+    for (int t = 0; t < 4; ++t)
+        for (int d = 0; d < 256; ++d) {
+            g64[(t * 256 + d) * 2] = T.Gre[t][d];
+            g64[(t * 256 + d) * 2 + 1] = T.Gim[t][d];
+        }
+    for (int k = 0; k < kK; ++k) {
+        g64[2048 + k] = pair_hidden(pairs, k) ? 0.0 : inv_or_zero(q[k], T.D[k]);
+        g64[2048 + kK + k] = inv_or_zero(1.0, T.D[k]);
+    }
+}
+
 void build_record64(const uint8_t *key, const double *w, const Cd *r32, uint32_t slot_ap, bool pairs,
-                    const std::vector<double> &q, Record<double> *rec)
+                    const std::vector<double> &q, Record<double> *rec, double *g64)
 {
     static thread_local Tables T;
     build_tables(key, w, r32, slot_ap, T);
+    if (g64) build_tables64(T, pairs, q, g64);
     for (int d = 0; d < 256; ++d) {
         rec->G01[d] = {T.Gre[0][d], T.Gim[0][d], T.Gre[1][d], T.Gim[1][d]};
         rec->G23[d] = {T.Gre[2][d], T.Gim[2][d], T.Gre[3][d], T.Gim[3][d]};
@@ -176,17 +191,7 @@ void build_record32(const uint8_t *key, const double *w, const Cd *r32, uint32_t
 {
     static thread_local Tables T;
     build_tables(key, w, r32, slot_ap, T);
-    if (g64) {   // FP64 tables for the stored Gram matrix: G_t [t][d] as (re, im), q/D, 1/D
-        for (int t = 0; t < 4; ++t)
-            for (int d = 0; d < 256; ++d) {
-                g64[(t * 256 + d) * 2] = T.Gre[t][d];
-                g64[(t * 256 + d) * 2 + 1] = T.Gim[t][d];
-            }
-        for (int k = 0; k < kK; ++k) {
-            g64[2048 + k] = pair_hidden(pairs, k) ? 0.0 : inv_or_zero(q[k], T.D[k]);
-            g64[2048 + kK + k] = inv_or_zero(1.0, T.D[k]);
-        }
-    }
+    if (g64) build_tables64(T, pairs, q, g64);
     for (int d = 0; d < 256; ++d) {
         float *a = sh->G01[d], *b = sh->G23[d];
         a[0] = (float)T.Gre[0][d]; a[1] = (float)T.Gre[1][d]; a[2] = (float)T.Gim[0][d]; a[3] = (float)T.Gim[1][d];
@@ -465,7 +470,16 @@ int create(rljsde_plan **out, int n_images, const uint8_t *const *masks, const i
     // Table sets whose Gram matrix is stored (c_supply): all of them (1),
     // those at least kStoredMinBlocks blocks use (3), or (auto) all, the most
     // used first, within an eighth of the free device memory.
-    if (!p->direct && !p->onthefly && prm->precision == 0 && prm->c_supply != 2 && foldable) {
+    // FP64 plans store FP64 matrices by the same rule (auto; not for the pair
+    // update, which keeps the factored loop) if one pass earns the build back:
+    // a table set takes about 47 us to build and a block-iteration is at least
+    // 0.18 us (64x64, latency bound) or 0.043 us (256x256) faster; measured,
+    // plan and one pass at nu_max 100, stored / factored: 64x64 6.5 / 6.5 ms,
+    // 128x128 7.1 / 12.1, 256x256 11.3 / 24.1.  Their state is R, so any q will do.
+    const size_t table_bytes = prm->precision ? kStored64Bytes : kStoredTableBytes;
+    const bool can_store =
+        prm->precision ? prm->pairs == 0 && total_blocks * prm->nu_max >= 250ll * p->n_tables : foldable;
+    if (!p->direct && !p->onthefly && prm->c_supply != 2 && can_store) {
         p->cslot.assign(p->n_tables, -1);
         if (prm->c_supply != 0) {
             for (int t = 0; t < p->n_tables; ++t) {
@@ -481,7 +495,7 @@ int create(rljsde_plan **out, int n_images, const uint8_t *const *masks, const i
             for (int t = 0; t < p->n_tables; ++t) order[t] = t;
             std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return count[x] > count[y]; });
             for (int t : order) {
-                if ((size_t)(p->n_stored + 1) * kStoredTableBytes > budget) break;
+                if ((size_t)(p->n_stored + 1) * table_bytes > budget) break;
                 p->cslot[t] = p->n_stored++;
                 p->n_stored_blocks += count[t];
             }
@@ -533,7 +547,10 @@ int create(rljsde_plan **out, int n_images, const uint8_t *const *masks, const i
                 const uint8_t *key = (const uint8_t *)keys[t].data();
                 if (prm->precision)
                     build_record64(key, w64, r32, slot_ap, prm->pairs != 0, p->q,
-                                   (Record<double> *)(host.data() + p->record_bytes * t));
+                                   (Record<double> *)(host.data() + p->record_bytes * t),
+                                   p->n_stored && p->cslot[t] >= 0
+                                       ? g64.data() + (size_t)kStoredBuildDoubles * p->cslot[t]
+                                       : nullptr);
                 else
                     build_record32(key, w64, r32, slot_ap, prm->pairs != 0, p->q,
                                    (RecordF32 *)(host.data() + p->record_bytes * t),
@@ -548,7 +565,7 @@ int create(rljsde_plan **out, int n_images, const uint8_t *const *masks, const i
             if (!st && p->n_stored) {
                 // the Gram matrices (Eq. 14) of the stored table sets, built on the device
                 double *d_g64 = nullptr;
-                p->cstore_bytes = kStoredTableBytes * (size_t)p->n_stored;
+                p->cstore_bytes = table_bytes * (size_t)p->n_stored;
                 if (cudaMalloc(&p->d_cstore, p->cstore_bytes) != cudaSuccess) {
                     p->d_cstore = nullptr;
                     cudaGetLastError();
