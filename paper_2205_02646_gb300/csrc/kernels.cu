@@ -2072,38 +2072,105 @@ __global__ void __launch_bounds__(kFlyWarps * 32, 2) onthefly_kernel(const Args 
 }
 
 // ---------------------------------------------------------- direct path --
-// Direct L-JSDE (Eqs. 4-10): per block the residual r (256 complex, in the
-// warp's scratch) and, every iteration, N_k = sum_m conj(a_m(k)) w_m r_m for
-// all 1024 k with a_m(k) evaluated from the roots-of-unity table (O(W^4)).
-// Any per-pixel aperture: a_m(k) sums the phases of m's transparent
-// sub-pixels; a candidate whose phase sum cancels exactly for every aperture
-// in the window is not observed by any measurement and scores 0.
+// Direct L-JSDE (Eqs. 4-10): per block the residual r (256 complex, in shared
+// memory) and, every iteration, N_k = sum_m conj(a_m(k)) w_m r_m for all 1024
+// k with a_m(k) evaluated from the roots-of-unity table (O(W^4)).  Any
+// per-pixel aperture: a_m(k) sums the phases of m's transparent sub-pixels; a
+// candidate whose phase sum cancels exactly for every aperture in the window
+// is not observed by any measurement and scores 0.
+//
+// One CTA of four warps per block (a warp per block left most schedulers
+// idle on the small images this path serves).  A thread holds two groups of
+// four candidates (k1 + 16 A, k2 + 16 B): their phases at a sub-pixel (dy, dx)
+// differ only in sign, (-1)^(A dy + B dx), and the table's entry n + 16 is
+// exactly the negative of entry n, so one lookup serves four candidates.  The
+// loop over the window branches to code specialised on the aperture.  Bound by
+// issue: about 11 instructions per candidate and measurement (20 before).
+// 96x64 HR, 15 apertures, nu_max 100: 19.4 -> 6.0 ms.
 constexpr int kDirectWarps = 4;
 struct DirectSmem {
-    float2 r[kDirectWarps][256];
-    float wr[kDirectWarps][256][2];
-    uint8_t type[kDirectWarps][256];     // aperture code, 0 = no measurement
+    float4 x[256];                        // w r (re, im), aperture code, weight
+    float2 r[256];
     float2 om[32];
     float w[256];
+    float4 best[kDirectWarps];            // score, candidate, N / D (re, im)
 };
+
+// One measurement's terms for a thread's eight candidates: add(j, A, B, are, aim)
+// with a_m(k) at k = (k1 + j + 16 A, k2 + 16 B); o1 = 2 p, o2 = 2 q.
+template <int AP, typename Add>
+__device__ __forceinline__ void direct_terms(const float2 *om, const int o1, const int o2, const int k1, const int k2,
+                                             Add add)
+{
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        float2 z[4];
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+            if ((AP >> s) & 1) z[s] = om[((o1 + (s >> 1)) * (k1 + j) + (o2 + (s & 1)) * k2) & 31];
+#pragma unroll
+        for (int A = 0; A < 2; ++A)
+#pragma unroll
+            for (int B = 0; B < 2; ++B) {
+                float are = 0.f, aim = 0.f;
+#pragma unroll
+                for (int s = 0; s < 4; ++s) {
+                    if (!((AP >> s) & 1)) continue;
+                    const bool neg = ((A & (s >> 1)) ^ (B & (s & 1))) != 0;
+                    are += neg ? -z[s].x : z[s].x;
+                    aim += neg ? -z[s].y : z[s].y;
+                }
+                add(j, A, B, are, aim);
+            }
+    }
+}
+template <typename Add>
+__device__ __forceinline__ void direct_measurement(const int ap, const float2 *om, const int m, const int k1, const int k2,
+                                                   Add add)
+{
+    const int o1 = 2 * (m >> 4), o2 = 2 * (m & 15);
+    switch (ap) {
+    case 1: direct_terms<1>(om, o1, o2, k1, k2, add); break;
+    case 2: direct_terms<2>(om, o1, o2, k1, k2, add); break;
+    case 3: direct_terms<3>(om, o1, o2, k1, k2, add); break;
+    case 4: direct_terms<4>(om, o1, o2, k1, k2, add); break;
+    case 5: direct_terms<5>(om, o1, o2, k1, k2, add); break;
+    case 6: direct_terms<6>(om, o1, o2, k1, k2, add); break;
+    case 7: direct_terms<7>(om, o1, o2, k1, k2, add); break;
+    case 8: direct_terms<8>(om, o1, o2, k1, k2, add); break;
+    case 9: direct_terms<9>(om, o1, o2, k1, k2, add); break;
+    case 10: direct_terms<10>(om, o1, o2, k1, k2, add); break;
+    case 11: direct_terms<11>(om, o1, o2, k1, k2, add); break;
+    case 12: direct_terms<12>(om, o1, o2, k1, k2, add); break;
+    case 13: direct_terms<13>(om, o1, o2, k1, k2, add); break;
+    case 14: direct_terms<14>(om, o1, o2, k1, k2, add); break;
+    case 15: direct_terms<15>(om, o1, o2, k1, k2, add); break;
+    default: break;                       // no measurement
+    }
+}
 
 __global__ void __launch_bounds__(kDirectWarps * 32) direct_kernel(const Args a, int n_entries)
 {
     __shared__ DirectSmem sm;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) sm.w[i] = a.consts->w32[i];
-    for (int i = threadIdx.x; i < 32; i += blockDim.x) sm.om[i] = make_float2(a.consts->om32[2 * i], a.consts->om32[2 * i + 1]);
-    __syncthreads();
+    __shared__ unsigned present_s;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int k2 = lane & 15, k1 = 8 * (lane >> 4) + 2 * warp;     // groups k1, k1 + 1
+    for (int i = tid; i < 256; i += blockDim.x) sm.w[i] = a.consts->w32[i];
+    for (int i = tid; i < 32; i += blockDim.x) sm.om[i] = make_float2(a.consts->om32[2 * i], a.consts->om32[2 * i + 1]);
     const float gamma = a.gamma32;
-    for (int e = blockIdx.x * kDirectWarps + warp; e < n_entries; e += gridDim.x * kDirectWarps) {
+    auto cand = [&](int j, int A, int B) { return (k1 + j + 16 * A) * kW + k2 + 16 * B; };
+    for (int e = blockIdx.x; e < n_entries; e += gridDim.x) {
         const WorkEntry we = a.entries[e];
         if (we.img < 0) continue;
         const ImageDesc img = a.descs ? a.descs[we.img] : a.single;
         const uint8_t *mask = a.masks + a.mask_offset[we.img];
         const int p0 = 2 * we.bi - kOff / 2, q0 = 2 * we.bj - kOff / 2;
+        __syncthreads();                  // the previous block is done with the shared arrays
+        if (tid == 0) present_s = 0;
+        __syncthreads();
         bool bad = false;
         uint32_t present = 0;                // bit a: aperture a occurs in the window
-        for (int m = lane; m < 256; m += 32) {
+        for (int m = tid; m < 256; m += blockDim.x) {
             const int p = m >> 4, q = m & 15, P = p0 + p, Q = q0 + q;
             int t = 0;
             float y = 0.f;
@@ -2116,102 +2183,96 @@ __global__ void __launch_bounds__(kDirectWarps * 32) direct_kernel(const Args a,
                 }
             }
             present |= 1u << t;
-            sm.type[warp][m] = (uint8_t)t;
-            sm.r[warp][m] = make_float2(y, 0.f);
+            sm.x[m] = make_float4(0.f, 0.f, __int_as_float(t), t != 0 ? sm.w[m] : 0.f);
+            sm.r[m] = make_float2(y, 0.f);
         }
         if (bad) atomicOr(a.status, kStatusNonfinite);
-        present = __reduce_or_sync(0xffffffffu, present) & ~1u;
-        __syncwarp();
-        // D_k = sum_m w_m |a_m(k)|^2 for this lane's 32 candidates k = lane + 32 j
-        float D[32];
-        for (int j = 0; j < 32; ++j) D[j] = 0.f;
+        present = __reduce_or_sync(0xffffffffu, present);
+        if (lane == 0) atomicOr(&present_s, present);
+        __syncthreads();
+        present = present_s & ~1u;
+        // D_k = sum_m w_m |a_m(k)|^2 for this thread's 8 candidates
+        float D[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) D[c] = 0.f;
+#pragma unroll 1
         for (int m = 0; m < 256; ++m) {
-            const int t = sm.type[warp][m];
-            if (t == 0) continue;
-            const int p = m >> 4, q = m & 15;
-            const float wm = sm.w[m];
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const int k1 = j, k2 = lane;
-                float are = 0.f, aim = 0.f;
-#pragma unroll
-                for (int s = 0; s < 4; ++s) {
-                    if (!((t >> s) & 1)) continue;
-                    const float2 z = sm.om[((2 * p + (s >> 1)) * k1 + (2 * q + (s & 1)) * k2) & 31];
-                    are += z.x;
-                    aim += z.y;
-                }
-                D[j] += wm * (are * are + aim * aim);
-            }
+            const float4 x = sm.x[m];
+            const float wm = x.w;
+            direct_measurement(__float_as_int(x.z), sm.om, m, k1, k2, [&](int j, int A, int B, float are, float aim) {
+                D[4 * j + 2 * A + B] += wm * (are * are + aim * aim);
+            });
         }
         // candidates no aperture of the window observes
 #pragma unroll
-        for (int j = 0; j < 32; ++j)
-            if ((present & ~(uint32_t)a.consts->vanish[j * kW + lane]) == 0) D[j] = 0.f;
+        for (int c = 0; c < 8; ++c)
+            if ((present & ~(uint32_t)a.consts->vanish[cand(c >> 2, (c >> 1) & 1, c & 1)]) == 0) D[c] = 0.f;
         float fpix = 0.f;
         const int eta = kOff + ((lane >> 2) & 3), gam = kOff + (lane & 3);
         const long long trow = (long long)we.ord * a.nu_max;
         for (int it = 0; it < a.nu_max; ++it) {
-            for (int m = lane; m < 256; m += 32) {
-                const float wm = sm.type[warp][m] != 0 ? sm.w[m] : 0.f;
-                sm.wr[warp][m][0] = wm * sm.r[warp][m].x;
-                sm.wr[warp][m][1] = wm * sm.r[warp][m].y;
+            for (int m = tid; m < 256; m += blockDim.x) {
+                const float wm = sm.x[m].w;
+                const float2 r = sm.r[m];
+                sm.x[m].x = wm * r.x;
+                sm.x[m].y = wm * r.y;
             }
-            __syncwarp();
-            float Nre[32], Nim[32];
-            for (int j = 0; j < 32; ++j) Nre[j] = Nim[j] = 0.f;
+            __syncthreads();
+            float Nre[8], Nim[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) Nre[c] = Nim[c] = 0.f;
+#pragma unroll 1
             for (int m = 0; m < 256; ++m) {
-                const int t = sm.type[warp][m];
-                if (t == 0) continue;
-                const int p = m >> 4, q = m & 15;
-                const float xr = sm.wr[warp][m][0], xi = sm.wr[warp][m][1];
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    float are = 0.f, aim = 0.f;
-#pragma unroll
-                    for (int s = 0; s < 4; ++s) {
-                        if (!((t >> s) & 1)) continue;
-                        const float2 z = sm.om[((2 * p + (s >> 1)) * j + (2 * q + (s & 1)) * lane) & 31];
-                        are += z.x;
-                        aim += z.y;
-                    }
+                const float4 x = sm.x[m];
+                const float xr = x.x, xi = x.y;
+                direct_measurement(__float_as_int(x.z), sm.om, m, k1, k2, [&](int j, int A, int B, float are, float aim) {
+                    const int c = 4 * j + 2 * A + B;
                     // conj(a) * (w r)
-                    Nre[j] += are * xr + aim * xi;
-                    Nim[j] += are * xi - aim * xr;
-                }
+                    Nre[c] += are * xr + aim * xi;
+                    Nim[c] += are * xi - aim * xr;
+                });
             }
             float bs = -1.f;
-            int bk = 0;
+            int bk = kK;
             float bre = 0.f, bim = 0.f;
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const int k = j * kW + lane;
+            for (int c = 0; c < 8; ++c) {
+                const int k = cand(c >> 2, (c >> 1) & 1, c & 1);
                 // conjugate-pair update: the argmax sees one member of each pair
-                if (a.pairs && ((-j) & 31) * kW + ((-lane) & 31) < k) continue;
-                const float s = D[j] > 0.f ? a.q[k] * (Nre[j] * Nre[j] + Nim[j] * Nim[j]) / D[j] : 0.f;
-                if (s > bs) {
+                if (a.pairs && mirror_of(k) < k) continue;
+                const float s = D[c] > 0.f ? a.q[k] * (Nre[c] * Nre[c] + Nim[c] * Nim[c]) / D[c] : 0.f;
+                if (s > bs || (s == bs && k < bk)) {
                     bs = s;
                     bk = k;
-                    bre = D[j] > 0.f ? Nre[j] / D[j] : 0.f;
-                    bim = D[j] > 0.f ? Nim[j] / D[j] : 0.f;
+                    bre = D[c] > 0.f ? Nre[c] / D[c] : 0.f;
+                    bim = D[c] > 0.f ? Nim[c] / D[c] : 0.f;
                 }
             }
+            const int own = bk;
 #pragma unroll
             for (int m = 16; m >= 1; m >>= 1) {
                 const float os = __shfl_xor_sync(0xffffffffu, bs, m);
                 const int ok = __shfl_xor_sync(0xffffffffu, bk, m);
                 if (os > bs || (os == bs && ok < bk)) { bs = os; bk = ok; }
             }
-            const int wl = bk & 31;
-            const float dre = __shfl_sync(0xffffffffu, bre, wl), dim = __shfl_sync(0xffffffffu, bim, wl);
-            const float gre = gamma * dre, gim = gamma * dim;
-            const int u = bk >> 5, v = bk & 31;
+            if (own == bk && own < kK) sm.best[warp] = make_float4(bs, __int_as_float(bk), bre, bim);
+            else if (lane == 0 && bk >= kK) sm.best[warp] = make_float4(-1.f, __int_as_float(kK), 0.f, 0.f);
+            __syncthreads();
+            float4 win = sm.best[0];
+#pragma unroll
+            for (int w = 1; w < kDirectWarps; ++w) {
+                const float4 o = sm.best[w];
+                if (o.x > win.x || (o.x == win.x && __float_as_int(o.y) < __float_as_int(win.y))) win = o;
+            }
+            const int uv = __float_as_int(win.y) & (kK - 1);
+            const float gre = gamma * win.z, gim = gamma * win.w;
+            const int u = uv >> 5, v = uv & 31;
             // conjugate-pair update: c_-uv += conj(gamma delta) as well (not for uv = -uv),
             // so r -= x + conj(x) with x = gamma delta a_m(uv): twice its real part
             const float pf = (a.pairs && ((u & 15) != 0 || (v & 15) != 0)) ? 2.f : 1.f;
             // r_m -= gamma delta a_m(uv)   (Eq. 7)
-            for (int m = lane; m < 256; m += 32) {
-                const int t = sm.type[warp][m];
+            for (int m = tid; m < 256; m += blockDim.x) {
+                const int t = __float_as_int(sm.x[m].z);
                 if (t == 0) continue;
                 const int p = m >> 4, q = m & 15;
                 float are = 0.f, aim = 0.f;
@@ -2221,29 +2282,29 @@ __global__ void __launch_bounds__(kDirectWarps * 32) direct_kernel(const Args a,
                     are += z.x;
                     aim += z.y;
                 }
-                float2 r = sm.r[warp][m];
+                float2 r = sm.r[m];
                 if (pf == 2.f) {
                     r.x -= 2.f * (gre * are - gim * aim);
                 } else {
                     r.x -= gre * are - gim * aim;
                     r.y -= gre * aim + gim * are;
                 }
-                sm.r[warp][m] = r;
+                sm.r[m] = r;
             }
             const float2 ph = sm.om[(eta * u + gam * v) & 31];
             fpix += pf * (gre * ph.x - gim * ph.y);
-            if (a.trace_sel && lane == 0) {
-                a.trace_sel[trow + it] = (uint16_t)bk;
+            if (a.trace_sel && tid == 0) {
+                a.trace_sel[trow + it] = (uint16_t)uv;
                 a.trace_dc[2 * (trow + it)] = gre;
                 a.trace_dc[2 * (trow + it) + 1] = gim;
             }
-            __syncwarp();
+            // (each thread weights the entries of r it has just written; the next
+            // barrier separates them, and best, from their other readers)
         }
-        if (lane < 16) {
-            const int yy = 4 * we.bi + (lane >> 2), xx = 4 * we.bj + (lane & 3);
+        if (tid < 16) {
+            const int yy = 4 * we.bi + (tid >> 2), xx = 4 * we.bj + (tid & 3);
             img.hr[(long long)yy * img.hr_pitch + xx] = fpix;
         }
-        __syncwarp();
     }
 }
 
@@ -2583,9 +2644,8 @@ int choose_launch(rljsde_plan *p, int warps, int ctas_per_sm)
         p->warps = kDirectWarps;
         p->ctas_per_sm = ctas_per_sm > 0 ? (ctas_per_sm < n ? ctas_per_sm : n) : n;
         if (p->ctas_per_sm < 1) p->ctas_per_sm = 1;
-        long long want = ((long long)p->n_entries + kDirectWarps - 1) / kDirectWarps;
         long long g = (long long)p->sm_count * p->ctas_per_sm;
-        p->grid = (int)(want < g ? (want > 0 ? want : 1) : g);
+        p->grid = (int)(p->n_entries < g ? (p->n_entries > 0 ? p->n_entries : 1) : g);
         return RLJSDE_OK;
     }
     // Default: 4 warps per CTA, as many CTAs as the 168-register variant fits.
