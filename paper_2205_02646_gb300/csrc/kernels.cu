@@ -850,7 +850,11 @@ struct Scan {
         t2 = p ? s2 : t2;
         bs = m;
     }
-    __device__ __forceinline__ int slot() const { return base + (t0 == bs ? 0 : t1 == bs ? 1 : t2 == bs ? 2 : 3); }
+    __device__ __forceinline__ int slot() const
+    {
+        const int lo = t0 == bs ? base : base + 1, hi = t2 == bs ? base + 2 : base + 3;
+        return t0 == bs || t1 == bs ? lo : hi;
+    }
 };
 
 // R of this lane's candidate in a slot (the same slot in every lane).
@@ -1048,15 +1052,30 @@ __device__ __forceinline__ void stored_block(const Args &a, const float4 *cs, co
     stored_setup<LAY>(a, cs, types, scratch, om, omc, pt, wt, we, lane, R);
     const int eta = kOff + ((lane >> 2) & 3), gam = kOff + (lane & 3);
     float fpix = 0.f;
-    for (int it = 0; it < a.nu_max; ++it) {
+    const int last = a.nu_max - 1;
+    auto trace = [&](const int it, const int bk, const C2<float> gd) {
+        if constexpr (TRACE) {
+            if (lane == 0) {
+                const long long row = (long long)we.ord * a.nu_max + it;
+                a.trace_sel[row] = (uint16_t)bk;
+                a.trace_dc[2 * row] = gd.re;
+                a.trace_dc[2 * row + 1] = gd.im;
+            }
+        }
+    };
+    // the last iteration, which updates nothing, is peeled: with the column
+    // loads and the update under a condition the loop spilled (1024x1024, nu_max
+    // 100: 2.82 -> 2.67 ms).  The mirrored loop has registers to spare and is
+    // faster with the condition (64x64 82 against 88 us).
+    for (int it = 0; it < (MIRROR ? last + 1 : last); ++it) {
+        const bool more = !MIRROR || it < last;
         const int bk = stored_argmax(R, lane);
-        const bool more = it + 1 < a.nu_max;
-        // column uv, or -uv to be read conjugated with the pairs' places exchanged
+        // column uv, or -uv to be read conjugated with the pairs' places
+        // exchanged; in flight during the bookkeeping
         const int mk = mirror_of(bk);
         const bool mir = MIRROR && mk < bk;
         float4 col[16];
         if (more) {
-            // in flight during the bookkeeping
             if (!mir) {
                 load_column(cs, bk, lane, col);
             } else {
@@ -1068,14 +1087,7 @@ __device__ __forceinline__ void stored_block(const Args &a, const float4 *cs, co
             }
         }
         const C2<float> gd = stored_step(R, bk, ldg_stream1(stored_invd(cs) + bk), a.gamma32, om, eta, gam, fpix);
-        if constexpr (TRACE) {
-            if (lane == 0) {
-                const long long row = (long long)we.ord * a.nu_max + it;
-                a.trace_sel[row] = (uint16_t)bk;
-                a.trace_dc[2 * row] = gd.re;
-                a.trace_dc[2 * row + 1] = gd.im;
-            }
-        }
+        trace(it, bk, gd);
         if (more) {
             const float2 ncre = f2(-gd.re, -gd.re), ncim = f2(-gd.im, -gd.im);
             float2 aim = ncre, are = f2(gd.im, gd.im);
@@ -1088,16 +1100,20 @@ __device__ __forceinline__ void stored_block(const Args &a, const float4 *cs, co
             for (int i = 0; i < 16; ++i) sub_pair(R[i], col[i], ncre, ncim, are, aim);
         }
     }
+    if constexpr (!MIRROR) {
+        const int bk = stored_argmax(R, lane);
+        trace(last, bk, stored_step(R, bk, ldg_stream1(stored_invd(cs) + bk), a.gamma32, om, eta, gam, fpix));
+    }
     store_pixel(a, we, lane, fpix);
 }
 
-// The same with the conjugate-pair update (1024x1024, nu_max 50: 2.65 -> 1.49
+// The same with the conjugate-pair update (1024x1024, nu_max 50: 2.65 -> 1.35
 // ms against updating all 1024 candidates from two columns).  The argmax runs
 // over k <= -k only: slots 1..15 of every lane and slots 0 and 16 of lanes
 // 0..16, so only those are kept and updated.  C_{k,-uv} = conj(C_{-k,uv}), and -k's rows are
 // scaled like k's in these plans, so one column serves both members of the
 // pair: 17 loads and 9 register pairs an iteration instead of 32 and 32.
-template <int LAY>
+template <int LAY, bool TRACE>
 __device__ __forceinline__ void stored_block_pairs(const Args &a, const float4 *cs, const uint8_t *types,
                                                    C2<float> *scratch, const C2<float> *om, const C2<float> *omc,
                                                    const PairTables &pt, const float *wt, const WorkEntry we,
@@ -1113,68 +1129,73 @@ __device__ __forceinline__ void stored_block_pairs(const Args &a, const float4 *
         if (hid) R[0] = {f2(0.f, 0.f), f2(0.f, 0.f)};
         R[8].re.y = R[8].im.y = 0.f;
     }
-    const float *invd = reinterpret_cast<const float *>(cs + kStoredInvDOff);
     const float gamma = a.gamma32;
     const int eta = kOff + ((lane >> 2) & 3), gam = kOff + (lane & 3);
     float fpix = 0.f, pw = 0.f;
-    int u = 0, v = 0;
-    C2<float> g[4];
-    const long long trow = (long long)we.ord * a.nu_max;
-
-    for (int it = 0; it < a.nu_max; ++it) {
+    const int last = a.nu_max - 1;
+    auto argmax = [&]() {
         Scan scan;
         scan.init();
-        {
-            float2 p[9];
+        float2 p[9];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) p[i] = norm2(R[i]);
-            scan.group<0>(p[0].x, p[1].x, p[1].y, p[2].x);
-            scan.group<4>(p[2].y, p[3].x, p[3].y, p[4].x);
-            scan.group<8>(p[4].y, p[5].x, p[5].y, p[6].x);
-            scan.group<12>(p[6].y, p[7].x, p[7].y, p[8].x);
-            scan.group<16>(p[0].y, 0.f, 0.f, 0.f);
-        }
+        for (int i = 0; i < 9; ++i) p[i] = norm2(R[i]);
+        scan.group<0>(p[0].x, p[1].x, p[1].y, p[2].x);
+        scan.group<4>(p[2].y, p[3].x, p[3].y, p[4].x);
+        scan.group<8>(p[4].y, p[5].x, p[5].y, p[6].x);
+        scan.group<12>(p[6].y, p[7].x, p[7].y, p[8].x);
+        scan.group<16>(p[0].y, 0.f, 0.f, 0.f);
         float bs = scan.bs;
         int bk = slot_k(scan.slot(), lane);
         warp_argmax(bs, bk);
-        const bool more = it + 1 < a.nu_max;
-        float4 own[9], mir[8];
-        if (more) {
-            const float4 *p = cs + (size_t)bk * 512 + lane;
-#pragma unroll
-            for (int i = 0; i < 9; ++i) own[i] = ldg_stream4(p + 32 * i);
-            mir[0] = ldg_stream4(cs + (size_t)bk * 512 + ((32 - lane) & 31));
-#pragma unroll
-            for (int i = 1; i < 8; ++i) mir[i] = ldg_stream4(p + 32 * (i + 8));
-            if (hid) own[0] = mir[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        const float invD = ldg_stream1(invd + bk);
-        const int wl = lane_of(bk), slot = bk >> 5;
+        return bk;
+    };
+    auto step = [&](const int it, const int bk, const float invD) {
         float mre, mim;
-        r_at_slot(R, slot, mre, mim);
-        const float Rre = __shfl_sync(0xffffffffu, mre, wl);
-        const float Rim = __shfl_sync(0xffffffffu, mim, wl);
-        select_step<float, LAY, true>(a, om, invD, gamma, bk, Rre, Rim, eta, gam, lane, trow, it, u, v, g, fpix, pw);
-        if (more) {
-            const C2<float> gd = {gamma * (Rre * invD), gamma * (Rim * invD)};   // as in select_step
-            const float2 ncre = f2(-gd.re, -gd.re), ncim = f2(-gd.im, -gd.im), cim = f2(gd.im, gd.im);
-            // the partner -uv gets pw conj(gamma delta) times the conjugate of the mirrored rows
-            const C2<float> pd = {pw * gd.re, -pw * gd.im};
-            const float2 npre = f2(-pd.re, -pd.re), npim = f2(-pd.im, -pd.im), pre = f2(pd.re, pd.re);
-            const float4 m8 = make_float4(own[8].y, 0.f, own[8].w, 0.f);
-            own[8].y = own[8].w = 0.f;
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                sub_pair(R[i], own[i], ncre, ncim, cim, ncre);
-                sub_pair(R[i], i < 8 ? mir[i & 7] : m8, npre, npim, npim, pre);
+        r_at_slot(R, bk >> 5, mre, mim);
+        const float Rre = __shfl_sync(0xffffffffu, mre, lane_of(bk));
+        const float Rim = __shfl_sync(0xffffffffu, mim, lane_of(bk));
+        int u, v;
+        C2<float> g[4];
+        const C2<float> gd = {gamma * (Rre * invD), gamma * (Rim * invD)};   // as in select_step
+        Args quiet = a;
+        quiet.trace_sel = nullptr;
+        select_step<float, LAY, true>(quiet, om, invD, gamma, bk, Rre, Rim, eta, gam, lane, 0, it, u, v, g, fpix, pw);
+        if constexpr (TRACE) {
+            if (lane == 0) {
+                const long long row = (long long)we.ord * a.nu_max + it;
+                a.trace_sel[row] = (uint16_t)bk;
+                a.trace_dc[2 * row] = gd.re;
+                a.trace_dc[2 * row + 1] = gd.im;
             }
         }
+        return gd;
+    };
+    for (int it = 0; it < last; ++it) {
+        const int bk = argmax();
+        float4 own[9], mir[8];
+        const float4 *p = cs + (size_t)bk * 512 + lane;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) own[i] = ldg_stream4(p + 32 * i);
+        mir[0] = ldg_stream4(cs + (size_t)bk * 512 + ((32 - lane) & 31));
+#pragma unroll
+        for (int i = 1; i < 8; ++i) mir[i] = ldg_stream4(p + 32 * (i + 8));
+        if (hid) own[0] = mir[0] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const C2<float> gd = step(it, bk, ldg_stream1(stored_invd(cs) + bk));
+        const float2 ncre = f2(-gd.re, -gd.re), ncim = f2(-gd.im, -gd.im), cim = f2(gd.im, gd.im);
+        // the partner -uv gets pw conj(gamma delta) times the conjugate of the mirrored rows
+        const C2<float> pd = {pw * gd.re, -pw * gd.im};
+        const float2 npre = f2(-pd.re, -pd.re), npim = f2(-pd.im, -pd.im), pre = f2(pd.re, pd.re);
+        const float4 m8 = make_float4(own[8].y, 0.f, own[8].w, 0.f);
+        own[8].y = own[8].w = 0.f;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            sub_pair(R[i], own[i], ncre, ncim, cim, ncre);
+            sub_pair(R[i], i < 8 ? mir[i & 7] : m8, npre, npim, npim, pre);
+        }
     }
-    if (lane < 16) {
-        const ImageDesc img = a.descs ? a.descs[we.img] : a.single;
-        const int yy = 4 * we.bi + (lane >> 2), xx = 4 * we.bj + (lane & 3);
-        img.hr[(long long)yy * img.hr_pitch + xx] = fpix;
-    }
+    const int bk = argmax();
+    step(last, bk, ldg_stream1(stored_invd(cs) + bk));
+    store_pixel(a, we, lane, fpix);
 }
 
 // ------------------------------------------ restricted (shortlist) loop --
@@ -1704,7 +1725,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) recurrent_kernel(const Args 
 // The stored-C loop on the blocks of the stored table sets: one warp per
 // block, the warps of a CTA independent of each other (no table in shared
 // memory: the loop needs only the window's types, the column and the scales).
-// 4096x3072, nu_max 100: 36.2 -> 33.0 ms against chunks of 8 blocks behind a
+// 4096x3072, nu_max 100: 36.3 -> 31.6 ms against chunks of 8 blocks behind a
 // shared table slot, eight warps an SM.
 // With LEARNED, only the blocks the gate sends back: the CTA lists them, a
 // batch of its entries at a time, and its warps take them from the list.
@@ -1769,7 +1790,7 @@ __global__ void __launch_bounds__(stored_warps(KIND) * 32, 1) stored_kernel(cons
     };
     auto block = [&](const uint32_t e) {
         if constexpr (KIND == kSoloPairs)
-            stored_block_pairs<LAY>(a, cols(e), types(e), scratch, om, omc, *pt, wt, a.entries[e], lane);
+            stored_block_pairs<LAY, TRACE>(a, cols(e), types(e), scratch, om, omc, *pt, wt, a.entries[e], lane);
         else
             stored_block<LAY, KIND != kSolo, TRACE>(a, cols(e), types(e), scratch, om, omc, *pt, wt, a.entries[e], lane);
     };
@@ -2375,7 +2396,7 @@ template <int LAY>
 StoredFn stored_fn_of(const int kind, const bool trace)
 {
     switch (kind) {
-    case kSoloPairs: return stored_kernel<LAY, kSoloPairs, true>;     // looks at the trace pointer itself
+    case kSoloPairs: return trace ? stored_kernel<LAY, kSoloPairs, true> : stored_kernel<LAY, kSoloPairs, false>;
     case kSoloMirror: return trace ? stored_kernel<LAY, kSoloMirror, true> : stored_kernel<LAY, kSoloMirror, false>;
     default: return trace ? stored_kernel<LAY, kSolo, true> : stored_kernel<LAY, kSolo, false>;
     }
