@@ -169,7 +169,6 @@ struct Args {
 template <typename T, int MODE = 0> struct RecOf;
 template <int MODE> struct RecOf<float, MODE> { using type = RecordF32; };
 template <> struct RecOf<float, 1> { using type = RecordShortF32; };
-template <> struct RecOf<float, 17> { using type = RecordShortF32; };   // mode 1 with stored C
 template <int MODE> struct RecOf<double, MODE> { using type = Record<double>; };
 
 // Pair tables of the FP32 loop: for kap1 pair j, (cos, cos, sin, sin) of
@@ -1268,11 +1267,6 @@ __device__ __forceinline__ void shortlist_setup(const Args &a, const RecordShort
     // R0 of the candidates at positions lane and lane + 32: Y_t(kap) =
     // sum_p T_t(p, kap2) w16^-(p kap1) over the row DFTs of the window
     // (through the scratch, two types a pass).
-    C2<float> hw[2][4];
-#pragma unroll
-    for (int c = 0; c < 2; ++c)
-#pragma unroll
-        for (int t = 0; t < 4; ++t) hw[c][t] = h_of(om, kw[c], t);
     C2<float> acc[4][4];
     window_rows<float>(a, rec.types, scratch, omc, wt, we, lane, acc);
     Vec4<float> *tb = reinterpret_cast<Vec4<float> *>(scratch);
@@ -1293,7 +1287,8 @@ __device__ __forceinline__ void shortlist_setup(const Args &a, const RecordShort
                 y0 = cadd(y0, cmul(C2<float>{tv.x, tv.y}, tw));
                 y1 = cadd(y1, cmul(C2<float>{tv.z, tv.w}, tw));
             }
-            Rw[c] = cadd(Rw[c], cadd(cmul(cconj(hw[c][2 * pass]), y0), cmul(cconj(hw[c][2 * pass + 1]), y1)));
+            Rw[c] = cadd(Rw[c], cadd(cmul(cconj(h_of(om, kw[c], 2 * pass)), y0),
+                                     cmul(cconj(h_of(om, kw[c], 2 * pass + 1)), y1)));
         }
     }
     // position 16 s + (lane & 15) sits at lane (16 s + (lane & 15)) mod 32, entry s / 2
@@ -1340,14 +1335,10 @@ __device__ __forceinline__ int shortlist_iterations(const Args &a, const Shortli
 // The shortlist loop for up to two blocks (on[b]: block b is present), one
 // per half-warp.  All lanes take part in every shuffle and ballot; a half
 // whose block is absent or done only skips the update.
-// STORED: the column of C comes from the plan's stored Gram matrix cs (one
-// 16-byte load per candidate, gathered from the 8 KiB column) instead of
-// being rebuilt from the factored tables.
-template <bool STORED>
+// The column of C is rebuilt from the factored tables.
 __device__ __forceinline__ void shortlist_pair(const Args &a, const RecordShortF32 &rec, C2<float> *scratch,
                                                const C2<float> *om, const C2<float> *omc, const float *wt,
-                                               const WorkEntry (&we)[2], const bool (&on)[2], const int lane,
-                                               const float4 *cs)
+                                               const WorkEntry (&we)[2], const bool (&on)[2], const int lane)
 {
     const int hb = lane >> 4;
     HalfState st;
@@ -1368,17 +1359,6 @@ __device__ __forceinline__ void shortlist_pair(const Args &a, const RecordShortF
             shortlist_setup(a, rec, scratch, om, omc, wt, we[b], sl, lane, b, st);
             nu[b] = shortlist_iterations(a, sl);
         }
-    if constexpr (STORED) {
-        // the stored columns' scaled state R'_k = s_k R_k, s_k = sqrt(q_k / D_k)
-        // from the record's q / D, whose score is |R'_k|^2
-#pragma unroll
-        for (int pr = 0; pr < 2; ++pr) {
-            const float2 sk = f2(sqrtf(st.qd[pr].x), sqrtf(st.qd[pr].y));
-            st.Rre[pr] = mul2(st.Rre[pr], sk);
-            st.Rim[pr] = mul2(st.Rim[pr], sk);
-            st.qd[pr] = f2(1.f, 1.f);
-        }
-    }
     const int nu_h = hb == 0 ? nu[0] : nu[1];
     const int numax = nu[0] > nu[1] ? nu[0] : nu[1];
     const WorkEntry me = hb == 0 ? we[0] : we[1];
@@ -1395,10 +1375,8 @@ __device__ __forceinline__ void shortlist_pair(const Args &a, const RecordShortF
         // the candidates holding it
         float2 sc01 = fma2(st.Rim[0], st.Rim[0], mul2(st.Rre[0], st.Rre[0]));
         float2 sc23 = fma2(st.Rim[1], st.Rim[1], mul2(st.Rre[1], st.Rre[1]));
-        if constexpr (!STORED) {
-            sc01 = mul2(st.qd[0], sc01);
-            sc23 = mul2(st.qd[1], sc23);
-        }
+        sc01 = mul2(st.qd[0], sc01);
+        sc23 = mul2(st.qd[1], sc23);
         const unsigned sb[4] = {__float_as_uint(sc01.x), __float_as_uint(sc01.y), __float_as_uint(sc23.x),
                                 __float_as_uint(sc23.y)};
         int bk;
@@ -1420,33 +1398,9 @@ __device__ __forceinline__ void shortlist_pair(const Args &a, const RecordShortF
         const int wl = 16 * hb + (mine ? __ffs(mine) - 1 : 0);
         const float sre = st.kc[0] == bk ? st.Rre[0].x : st.kc[1] == bk ? st.Rre[0].y : st.kc[2] == bk ? st.Rre[1].x : st.Rre[1].y;
         const float sim = st.kc[0] == bk ? st.Rim[0].x : st.kc[1] == bk ? st.Rim[0].y : st.kc[2] == bk ? st.Rim[1].x : st.Rim[1].y;
-        float4 cv[4];
-        if (STORED && it < nu_h) {
-            // the candidates' entries of column bk, in flight during the bookkeeping
-            const float4 *col = cs + (size_t)(bk & (kK - 1)) * 512;
-#pragma unroll
-            for (int sl4 = 0; sl4 < 4; ++sl4) cv[sl4] = ldg_stream4(col + st.coff[sl4]);
-        }
         const float Rre = __shfl_sync(0xffffffffu, sre, wl);
         const float Rim = __shfl_sync(0xffffffffu, sim, wl);
-        if (STORED && it < nu_h) {
-            // delta = R'_uv / (s_uv D_uv): a plan storing every table set's
-            // Gram matrix keeps 1 / (s D) in the record's invD
-            const float invD = rec.invD[bk & (kK - 1)];
-            select_step<float>(a, om, invD, gamma, bk & (kK - 1), Rre, Rim, eta, gam, lane & 15, trow, it, u, v, g,
-                               fpix, unused_pw);
-            // Eq. 17 on the shortlist with the stored column, as the stored-C loop does
-            const C2<float> gd = {gamma * (Rre * invD), gamma * (Rim * invD)};   // as in select_step
-            const float2 ngr = f2(-gd.re, -gd.re), gi = f2(gd.im, gd.im), ngi = f2(-gd.im, -gd.im);
-#pragma unroll
-            for (int pr = 0; pr < 2; ++pr) {
-                const float4 A = cv[2 * pr], B = cv[2 * pr + 1];
-                const bool ea = (st.ce >> (2 * pr)) & 1, eb = (st.ce >> (2 * pr + 1)) & 1;
-                const float2 Cre = f2(ea ? A.y : A.x, eb ? B.y : B.x), Cim = f2(ea ? A.w : A.z, eb ? B.w : B.z);
-                st.Rre[pr] = fma2(Cim, gi, fma2(Cre, ngr, st.Rre[pr]));
-                st.Rim[pr] = fma2(Cre, ngi, fma2(Cim, ngr, st.Rim[pr]));
-            }
-        } else if (!STORED && it < nu_h) {
+        if (it < nu_h) {
             select_step<float>(a, om, rec.invD[bk & (kK - 1)], gamma, bk & (kK - 1), Rre, Rim, eta, gam, lane & 15,
                                trow, it, u, v, g, fpix, unused_pw);
             // Eq. 17 on the shortlist: R_k -= sum_t conj(h_t(k)) g_t G_t(uv - k), two
@@ -1495,6 +1449,121 @@ __device__ __forceinline__ void shortlist_pair(const Args &a, const RecordShortF
     }
 }
 
+// The same with the column of C read from the plan's stored Gram matrices: one
+// 16-byte load per candidate, gathered from the 8 KiB column of the block's
+// table set (tables and matrices are read through the L1, not staged).
+__device__ __forceinline__ void shortlist_stored(const Args &a, const uint32_t (&e)[2], const bool (&on)[2],
+                                                 C2<float> *scratch, const C2<float> *om, const C2<float> *omc,
+                                                 const float *wt, const int lane)
+{
+    const int hb = lane >> 4;
+    const WorkEntry we[2] = {a.entries[e[0]], a.entries[e[1]]};
+    HalfState st;
+    st.ce = 0;
+#pragma unroll
+    for (int sl4 = 0; sl4 < 4; ++sl4) {
+        st.kc[sl4] = 0;
+        st.coff[sl4] = 0;
+        if (sl4 < 2) st.Rre[sl4] = st.Rim[sl4] = st.qd[sl4] = f2(0.f, 0.f);
+    }
+    int nu[2] = {0, 0};
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+        if (on[b]) {
+            const Shortlist &sl = a.shortlists[we[b].ord];
+            const RecordShortF32 &rec = reinterpret_cast<const RecordShortF32 *>(a.records_short)[a.chunk_table[e[b] / kChunk]];
+            shortlist_setup(a, rec, scratch, om, omc, wt, we[b], sl, lane, b, st);
+            nu[b] = shortlist_iterations(a, sl);
+        }
+    // the stored columns' scaled state R'_k = s_k R_k, s_k = sqrt(q_k / D_k)
+    // from the record's q / D, whose score is |R'_k|^2
+    unsigned key[4];                     // candidate, lane in the half, slot
+#pragma unroll
+    for (int pr = 0; pr < 2; ++pr) {
+        const float2 sk = f2(sqrtf(st.qd[pr].x), sqrtf(st.qd[pr].y));
+        st.Rre[pr] = mul2(st.Rre[pr], sk);
+        st.Rim[pr] = mul2(st.Rim[pr], sk);
+    }
+#pragma unroll
+    for (int sl4 = 0; sl4 < 4; ++sl4) key[sl4] = (unsigned)(st.kc[sl4] << 6 | (lane & 15) << 2 | sl4);
+    const int nu_h = hb == 0 ? nu[0] : nu[1];
+    const int numax = nu[0] > nu[1] ? nu[0] : nu[1];
+    const uint32_t tab = a.chunk_table[(hb == 0 ? e[0] : e[1]) / kChunk];
+    const float4 *cs = a.cstore + (size_t)a.cslot[tab] * (kStoredTableBytes / 16);
+    const float *invd = reinterpret_cast<const RecordShortF32 *>(a.records_short)[tab].invD;   // 1 / (s D)
+    const float gamma = a.gamma32;
+    const int eta = kOff + ((lane >> 2) & 3), gam = kOff + (lane & 3);
+    float fpix = 0.f;
+    const long long trow = (long long)(hb == 0 ? we[0].ord : we[1].ord) * a.nu_max;
+    for (int it = 0; it < numax; ++it) {
+        // scores of the four candidates (two f32x2 pairs), the half-warp's
+        // largest by warp reductions over each half's inputs (non-negative,
+        // so the bits order like the values), then the smallest candidate
+        // holding it, with where it is held
+        const float2 sc01 = fma2(st.Rim[0], st.Rim[0], mul2(st.Rre[0], st.Rre[0]));
+        const float2 sc23 = fma2(st.Rim[1], st.Rim[1], mul2(st.Rre[1], st.Rre[1]));
+        const unsigned sb[4] = {__float_as_uint(sc01.x), __float_as_uint(sc01.y), __float_as_uint(sc23.x),
+                                __float_as_uint(sc23.y)};
+        const unsigned bits = max(max(sb[0], sb[1]), max(sb[2], sb[3]));
+        const unsigned m0 = __reduce_max_sync(0xffffffffu, hb == 0 ? bits : 0u);
+        const unsigned m1 = __reduce_max_sync(0xffffffffu, hb == 1 ? bits : 0u);
+        const unsigned mh = hb == 0 ? m0 : m1;
+        unsigned kmin = 0xffffffffu;
+#pragma unroll
+        for (int sl4 = 0; sl4 < 4; ++sl4) kmin = min(kmin, sb[sl4] == mh ? key[sl4] : 0xffffffffu);
+        const unsigned i0 = __reduce_min_sync(0xffffffffu, hb == 0 ? kmin : 0xffffffffu);
+        const unsigned i1 = __reduce_min_sync(0xffffffffu, hb == 1 ? kmin : 0xffffffffu);
+        const unsigned best = hb == 0 ? i0 : i1;
+        const int bk = (int)(best >> 6) & (kK - 1), at = (int)best & 3, wl = 16 * hb + ((int)(best >> 2) & 15);
+        float4 cv[4];
+        float invD = 0.f;
+        if (it < nu_h) {
+            // the candidates' entries of column bk, in flight during the bookkeeping
+            const float4 *col = cs + (size_t)bk * 512;
+            invD = ldg_stream1(invd + bk);
+#pragma unroll
+            for (int sl4 = 0; sl4 < 4; ++sl4) cv[sl4] = ldg_stream4(col + st.coff[sl4]);
+        }
+        const float sre = at == 0 ? st.Rre[0].x : at == 1 ? st.Rre[0].y : at == 2 ? st.Rre[1].x : st.Rre[1].y;
+        const float sim = at == 0 ? st.Rim[0].x : at == 1 ? st.Rim[0].y : at == 2 ? st.Rim[1].x : st.Rim[1].y;
+        const float Rre = __shfl_sync(0xffffffffu, sre, wl);
+        const float Rim = __shfl_sync(0xffffffffu, sim, wl);
+        if (it < nu_h) {
+            // delta = R'_uv / (s_uv D_uv) (Eqs. 15, 16), its share of Eq. 18, as select_step does it
+            const C2<float> gd = {gamma * (Rre * invD), gamma * (Rim * invD)};
+            const C2<float> ph = om[(eta * (bk >> 5) + gam * (bk & 31)) & 31];
+            fpix += gd.re * ph.re - gd.im * ph.im;
+            if (a.trace_sel != nullptr && (lane & 15) == 0) {
+                a.trace_sel[trow + it] = (uint16_t)bk;
+                a.trace_dc[2 * (trow + it)] = gd.re;
+                a.trace_dc[2 * (trow + it) + 1] = gd.im;
+            }
+            // Eq. 17 on the shortlist with the stored column, as the stored-C loop does
+            const float2 ngr = f2(-gd.re, -gd.re), gi = f2(gd.im, gd.im), ngi = f2(-gd.im, -gd.im);
+#pragma unroll
+            for (int pr = 0; pr < 2; ++pr) {
+                const float4 A = cv[2 * pr], B = cv[2 * pr + 1];
+                const bool ea = (st.ce >> (2 * pr)) & 1, eb = (st.ce >> (2 * pr + 1)) & 1;
+                const float2 Cre = f2(ea ? A.y : A.x, eb ? B.y : B.x), Cim = f2(ea ? A.w : A.z, eb ? B.w : B.z);
+                st.Rre[pr] = fma2(Cim, gi, fma2(Cre, ngr, st.Rre[pr]));
+                st.Rim[pr] = fma2(Cre, ngi, fma2(Cim, ngr, st.Rim[pr]));
+            }
+        }
+    }
+    if (hb == 0 ? on[0] : on[1]) {
+        if (a.trace_sel != nullptr && (lane & 15) == 0)
+            for (int it = nu_h; it < a.nu_max; ++it) {
+                a.trace_sel[trow + it] = 0xFFFF;
+                a.trace_dc[2 * (trow + it)] = 0.f;
+                a.trace_dc[2 * (trow + it) + 1] = 0.f;
+            }
+        const WorkEntry me = hb == 0 ? we[0] : we[1];
+        const ImageDesc img = a.descs ? a.descs[me.img] : a.single;
+        const int yy = 4 * me.bi + ((lane >> 2) & 3), xx = 4 * me.bj + (lane & 3);
+        img.hr[(long long)yy * img.hr_pitch + xx] = fpix;
+    }
+}
+
 __device__ __forceinline__ int shortlist_iterations(const Args &a, const Shortlist &sl)
 {
     if (!a.use_nu_hat) return a.nu_max;
@@ -1510,17 +1579,14 @@ __device__ __forceinline__ int shortlist_iterations(const Args &a, const Shortli
 // of one does not constrain the other.  3 and 4 = mode 0 for other sensor
 // layouts: slot apertures from a.slot_ap (3), or one sub-pixel per slot (4).
 // Bit 3 (kModePairs) added to modes 0, 3, 4: the conjugate-pair update.
-// Bit 4 (kModeStoredC) added to mode 1: the column of C read from the stored
-// Gram matrix instead of rebuilt from the factored tables (the full loop with
-// stored columns is stored_kernel).
+// (The loops that read stored Gram matrices are stored_kernel, shortlist_kernel
+// and stored64_kernel.)
 constexpr int kModePairs = 8;
-constexpr int kModeStoredC = 16;
 __host__ __device__ constexpr int lay_of(int mode)
 {
     return (mode & 7) == 3 ? kLayGeneral : (mode & 7) == 4 ? kLaySingle : kLayThreeQuarter;
 }
 __host__ __device__ constexpr bool pairs_of(int mode) { return (mode & kModePairs) != 0; }
-__host__ __device__ constexpr bool stored_of(int mode) { return (mode & kModeStoredC) != 0; }
 __host__ __device__ constexpr bool plain_of(int mode) { return (mode & 7) == 0 || (mode & 7) == 3 || (mode & 7) == 4; }
 __host__ __device__ constexpr int learned_of(int mode) { return (mode & 7) == 1 || (mode & 7) == 2 ? (mode & 7) : 0; }
 
@@ -1529,8 +1595,7 @@ template <int MODE> struct Loop<float, MODE> {
     using Rec = typename RecOf<float, MODE>::type;
     static __device__ __forceinline__ void run(const Args &a, const Rec &rec, C2<float> *scratch,
                                                const C2<float> *om, const C2<float> *omc, const PairTables &pt,
-                                               const float *wt, const WorkEntry we, const int lane,
-                                               const float4 *cs)
+                                               const float *wt, const WorkEntry we, const int lane)
     {
         if constexpr (plain_of(MODE)) {
             C2<float> Y[8][4];
@@ -1542,7 +1607,7 @@ template <int MODE> struct Loop<float, MODE> {
             if (a.n_restricted != nullptr && lane == 0) atomicAdd(a.n_restricted, 1);
             const WorkEntry w2[2] = {we, we};
             const bool on[2] = {true, false};
-            shortlist_pair<stored_of(MODE)>(a, rec, scratch, om, omc, wt, w2, on, lane, cs);
+            shortlist_pair(a, rec, scratch, om, omc, wt, w2, on, lane);
         } else {
             const Shortlist &sl = a.shortlists[we.ord];
             if (sl.missing <= a.max_missing) return;
@@ -1557,7 +1622,7 @@ template <int MODE> struct Loop<float, MODE> {
     static __device__ __forceinline__ void run_pair(const Args &a, const Rec &rec, C2<float> *scratch,
                                                     const C2<float> *om, const C2<float> *omc,
                                                     const PairTables &pt, const float *wt, const WorkEntry e0,
-                                                    const WorkEntry e1, const int lane, const float4 *cs)
+                                                    const WorkEntry e1, const int lane)
     {
         const bool r0 = e0.img >= 0 && a.shortlists[e0.ord].missing <= a.max_missing;
         const bool r1 = e1.img >= 0 && a.shortlists[e1.ord].missing <= a.max_missing;
@@ -1565,14 +1630,13 @@ template <int MODE> struct Loop<float, MODE> {
         if (a.n_restricted != nullptr && lane == 0) atomicAdd(a.n_restricted, (int)r0 + (int)r1);
         const WorkEntry w2[2] = {e0, e1};
         const bool on[2] = {r0, r1};
-        shortlist_pair<stored_of(MODE)>(a, rec, scratch, om, omc, wt, w2, on, lane, cs);
+        shortlist_pair(a, rec, scratch, om, omc, wt, w2, on, lane);
     }
 };
 template <int MODE> struct Loop<double, MODE> {
     static __device__ __forceinline__ void run(const Args &a, const Record<double> &rec, C2<double> *scratch,
                                                const C2<double> *om, const C2<double> *omc, const PairTables &,
-                                               const double *wt, const WorkEntry we, const int lane,
-                                               const float4 *)
+                                               const double *wt, const WorkEntry we, const int lane)
     {
         C2<double> Y[8][4];
         initial_projection<double>(a, rec.types, scratch, omc, wt, we, lane, Y);
@@ -1581,10 +1645,10 @@ template <int MODE> struct Loop<double, MODE> {
     static __device__ __forceinline__ void run_pair(const Args &a, const Record<double> &rec, C2<double> *scratch,
                                                     const C2<double> *om, const C2<double> *omc,
                                                     const PairTables &pt, const double *wt, const WorkEntry e0,
-                                                    const WorkEntry e1, const int lane, const float4 *)
+                                                    const WorkEntry e1, const int lane)
     {
-        if (e0.img >= 0) run(a, rec, scratch, om, omc, pt, wt, e0, lane, nullptr);
-        if (e1.img >= 0) run(a, rec, scratch, om, omc, pt, wt, e1, lane, nullptr);
+        if (e0.img >= 0) run(a, rec, scratch, om, omc, pt, wt, e0, lane);
+        if (e1.img >= 0) run(a, rec, scratch, om, omc, pt, wt, e1, lane);
     }
 };
 
@@ -1682,21 +1746,16 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) recurrent_kernel(const Args 
             parity ^= 1u << s;
             pending &= ~(1u << s);
         }
-        const float4 *cs = nullptr;           // this chunk's stored Gram matrix, if any
-        if constexpr (stored_of(MODE)) {
-            const int cl = a.cslot[a.chunk_table[c]];
-            if (cl >= 0) cs = a.cstore + (size_t)cl * (kStoredTableBytes / 16);
-        }
         if (!work) {
             // no block of this chunk in this mode
         } else if constexpr (learned_of(MODE) == 1 && WARPS * 2 == kChunk) {
             const WorkEntry e0 = a.entries[(size_t)c * kChunk + warp];
             const WorkEntry e1 = a.entries[(size_t)c * kChunk + warp + WARPS];
-            Loop<T, MODE>::run_pair(a, *slot(s), scratch, om, omc, *pt, wt, e0, e1, lane, cs);
+            Loop<T, MODE>::run_pair(a, *slot(s), scratch, om, omc, *pt, wt, e0, e1, lane);
         } else {
             for (int e = warp; e < kChunk; e += WARPS) {
                 const WorkEntry we = a.entries[(size_t)c * kChunk + e];
-                if (we.img >= 0) Loop<T, MODE>::run(a, *slot(s), scratch, om, omc, *pt, wt, we, lane, cs);
+                if (we.img >= 0) Loop<T, MODE>::run(a, *slot(s), scratch, om, omc, *pt, wt, we, lane);
             }
         }
         __syncthreads();                       // every warp is done with slot s
@@ -1822,6 +1881,46 @@ __global__ void __launch_bounds__(stored_warps(KIND) * 32, 1) stored_kernel(cons
                 block(list[i]);
             }
         }
+    }
+}
+
+// The shortlist loop with stored Gram matrices: two blocks per warp, warps
+// independent, three per scheduler at 168 registers (1024x1024, nu_max 100, a
+// tenth of the blocks gated back, the whole learned pass: 1.90 -> 1.70 ms
+// against chunks of 8 blocks behind staged tables; 16 and 20 warps spill in
+// the setup, 1.75 and 1.77 ms).
+constexpr int kShortWarps = 12;
+struct ShortSmem {
+    static constexpr size_t off_scratch = 0;                                     // kShortWarps x 4 KB
+    static constexpr size_t off_om = kShortWarps * 256 * 2 * sizeof(C2<float>);
+    static constexpr size_t off_omc = off_om + 32 * sizeof(C2<float>);
+    static constexpr size_t off_w = off_omc + 32 * sizeof(C2<float>);
+    static constexpr size_t bytes = off_w + 256 * sizeof(float);
+};
+
+__global__ void __launch_bounds__(kShortWarps * 32, 1) shortlist_kernel(const Args a)
+{
+    using L = ShortSmem;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    C2<float> *scratch = reinterpret_cast<C2<float> *>(smem + L::off_scratch) + warp * 512;
+    C2<float> *om = reinterpret_cast<C2<float> *>(smem + L::off_om);
+    C2<float> *omc = reinterpret_cast<C2<float> *>(smem + L::off_omc);
+    float *wt = reinterpret_cast<float *>(smem + L::off_w);
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) wt[i] = a.consts->w32[i];
+    for (int i = threadIdx.x; i < 32; i += blockDim.x) {
+        om[i] = {a.consts->om32[2 * i], a.consts->om32[2 * i + 1]};
+        omc[i] = {a.consts->om32[2 * i], -a.consts->om32[2 * i + 1]};
+    }
+    __syncthreads();
+    for (int i = 2 * (blockIdx.x * kShortWarps + warp); i < a.n_order; i += 2 * gridDim.x * kShortWarps) {
+        const bool two = i + 1 < a.n_order;
+        const uint32_t e[2] = {a.order[i], a.order[two ? i + 1 : i]};
+        const bool on[2] = {a.shortlists[a.entries[e[0]].ord].missing <= a.max_missing,
+                            two && a.shortlists[a.entries[e[1]].ord].missing <= a.max_missing};
+        if (!on[0] && !on[1]) continue;
+        if (a.n_restricted != nullptr && lane == 0) atomicAdd(a.n_restricted, (int)on[0] + (int)on[1]);
+        shortlist_stored(a, e, on, scratch, om, omc, wt, lane);
     }
 }
 
@@ -2347,7 +2446,6 @@ const Variant kVariants[] = {
     RLJSDE_VARIANT(float, 4, 3, 4), RLJSDE_VARIANT(float, 8, 2, 4), RLJSDE_VARIANT(double, 4, 1, 4),
     RLJSDE_VARIANT(float, 4, 3, 8), RLJSDE_VARIANT(float, 4, 3, 11), RLJSDE_VARIANT(float, 4, 3, 12),
     RLJSDE_VARIANT(double, 4, 1, 8), RLJSDE_VARIANT(double, 4, 1, 11), RLJSDE_VARIANT(double, 4, 1, 12),
-    RLJSDE_VARIANT(float, 4, 3, 17),
 };
 #undef RLJSDE_VARIANT
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
@@ -2747,14 +2845,18 @@ int rljsde_reconstruct_learned(const rljsde_plan_t *plan, const float *lr, size_
     a.n_restricted = n_restricted;
     // shortlist blocks first, then the full loop on the rest
     // with every table set's Gram matrix stored, both loops read its columns
-    const int sc = plan->n_stored > 0 && plan->n_stored == plan->n_tables ? kModeStoredC : 0;
-    const int lw = sc ? 4 : plan->learned_warps, lm = sc ? 3 : plan->learned_minb;
-    int st = launch_mode(plan, a, 1 | sc, lw, lm, (cudaStream_t)stream);
-    if (st == RLJSDE_OK && sc) {
-        st = launch_stored(plan, a, kFallback, (cudaStream_t)stream);
-    } else if (st == RLJSDE_OK) {
-        st = launch_mode(plan, a, 2, 4, 0, (cudaStream_t)stream);
+    if (plan->n_stored > 0 && plan->n_stored == plan->n_tables) {
+        if (cudaFuncSetAttribute(shortlist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ShortSmem::bytes) !=
+            cudaSuccess)
+            return RLJSDE_ERR_CUDA;
+        const int want = (plan->n_order + 2 * kShortWarps - 1) / (2 * kShortWarps);
+        shortlist_kernel<<<want < plan->sm_count ? want : plan->sm_count, kShortWarps * 32, ShortSmem::bytes,
+                           (cudaStream_t)stream>>>(a);
+        if (cudaGetLastError() != cudaSuccess) return RLJSDE_ERR_CUDA;
+        return launch_stored(plan, a, kFallback, (cudaStream_t)stream);
     }
+    int st = launch_mode(plan, a, 1, plan->learned_warps, plan->learned_minb, (cudaStream_t)stream);
+    if (st == RLJSDE_OK) st = launch_mode(plan, a, 2, 4, 0, (cudaStream_t)stream);
     return st;
 }
 
