@@ -1579,8 +1579,8 @@ __device__ __forceinline__ int shortlist_iterations(const Args &a, const Shortli
 // of one does not constrain the other.  3 and 4 = mode 0 for other sensor
 // layouts: slot apertures from a.slot_ap (3), or one sub-pixel per slot (4).
 // Bit 3 (kModePairs) added to modes 0, 3, 4: the conjugate-pair update.
-// (The loops that read stored Gram matrices are stored_kernel, shortlist_kernel
-// and stored64_kernel.)
+// (The loops that read stored Gram matrices are stored_kernel and
+// stored64_kernel.)
 constexpr int kModePairs = 8;
 __host__ __device__ constexpr int lay_of(int mode)
 {
@@ -1786,8 +1786,12 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) recurrent_kernel(const Args 
 // memory: the loop needs only the window's types, the column and the scales).
 // 4096x3072, nu_max 100: 36.3 -> 31.6 ms against chunks of 8 blocks behind a
 // shared table slot, eight warps an SM.
-// With LEARNED, only the blocks the gate sends back: the CTA lists them, a
-// batch of its entries at a time, and its warps take them from the list.
+// kLearned runs the learned path: the CTA lists its blocks the gate sends
+// back, a batch of its entries at a time, its warps take them from the list,
+// and a warp that finds the list empty goes on to the CTA's shortlisted
+// blocks, two at a time (in two kernels, one after the other, the full loop
+// had the SMs to itself while its last blocks ran: 1024x1024, nu_max 100,
+// a tenth of the blocks sent back: 1.72 -> 1.59 ms; 256x256: 381 -> 253 us).
 constexpr int kStoredWarps = 12;
 constexpr int kStoredBatch = 2048;
 struct StoredSmem {
@@ -1818,7 +1822,7 @@ __device__ __forceinline__ void fill_tables(const Args &a, C2<float> *om, C2<flo
     }
 }
 
-enum StoredKind { kSolo, kSoloMirror, kSoloPairs, kFallback, kFp64 };
+enum StoredKind { kSolo, kSoloMirror, kSoloPairs, kLearned, kFp64 };
 // Warps per CTA (one CTA per SM).  Twelve is three per scheduler at 168
 // registers: the loop is bound by the latency of its own instructions (issue
 // active 52 %, ALU and FMA pipes 42 %, no memory unit above 58 %), and the
@@ -1851,76 +1855,48 @@ __global__ void __launch_bounds__(stored_warps(KIND) * 32, 1) stored_kernel(cons
         if constexpr (KIND == kSoloPairs)
             stored_block_pairs<LAY, TRACE>(a, cols(e), types(e), scratch, om, omc, *pt, wt, a.entries[e], lane);
         else
-            stored_block<LAY, KIND != kSolo, TRACE>(a, cols(e), types(e), scratch, om, omc, *pt, wt, a.entries[e], lane);
+            stored_block<LAY, KIND == kSoloMirror, TRACE>(a, cols(e), types(e), scratch, om, omc, *pt, wt, a.entries[e], lane);
     };
-    if constexpr (KIND != kFallback) {
+    if constexpr (KIND != kLearned) {
         for (int i = blockIdx.x * warps + warp; i < a.n_order; i += gridDim.x * warps) block(a.order[i]);
     } else {
         __shared__ uint32_t list[kStoredBatch];
-        __shared__ int n_list, next;
+        __shared__ int n_list, next, next_pair;
         // entries o of this CTA: runs of kChunk, every gridDim-th run
         const long long runs = ((long long)a.n_order + kChunk - 1) / kChunk;
         const long long mine = ((runs - blockIdx.x + gridDim.x - 1) / gridDim.x) * kChunk;
+        auto entry = [&](const long long j) {             // this CTA's j-th place in the order, or beyond its end
+            return ((j / kChunk) * gridDim.x + blockIdx.x) * kChunk + j % kChunk;
+        };
+        auto taken = [&](int *counter) {                  // the next number for this warp
+            int i = 0;
+            if (lane == 0) i = atomicAdd(counter, 1);
+            return __shfl_sync(0xffffffffu, i, 0);
+        };
+        auto restricted = [&](const uint32_t e) { return a.shortlists[a.entries[e].ord].missing <= a.max_missing; };
+        if (threadIdx.x == 0) next_pair = 0;
         for (long long b0 = 0; b0 < mine; b0 += kStoredBatch) {
             __syncthreads();
             if (threadIdx.x == 0) n_list = next = 0;
             __syncthreads();
             for (int i = threadIdx.x; i < kStoredBatch && b0 + i < mine; i += blockDim.x) {
-                const long long j = b0 + i;
-                const long long o = ((j / kChunk) * gridDim.x + blockIdx.x) * kChunk + j % kChunk;
-                if (o >= a.n_order) continue;
-                const uint32_t e = a.order[o];
-                if (!(a.shortlists[a.entries[e].ord].missing <= a.max_missing)) list[atomicAdd(&n_list, 1)] = e;
+                const long long o = entry(b0 + i);
+                if (o < a.n_order && !restricted(a.order[o])) list[atomicAdd(&n_list, 1)] = a.order[o];
             }
             __syncthreads();
-            for (;;) {
-                int i = 0;
-                if (lane == 0) i = atomicAdd(&next, 1);
-                i = __shfl_sync(0xffffffffu, i, 0);
-                if (i >= n_list) break;
-                block(list[i]);
-            }
+            for (int i = taken(&next); i < n_list; i = taken(&next)) block(list[i]);
         }
-    }
-}
-
-// The shortlist loop with stored Gram matrices: two blocks per warp, warps
-// independent, three per scheduler at 168 registers (1024x1024, nu_max 100, a
-// tenth of the blocks gated back, the whole learned pass: 1.90 -> 1.70 ms
-// against chunks of 8 blocks behind staged tables; 16 and 20 warps spill in
-// the setup, 1.75 and 1.77 ms).
-constexpr int kShortWarps = 12;
-struct ShortSmem {
-    static constexpr size_t off_scratch = 0;                                     // kShortWarps x 4 KB
-    static constexpr size_t off_om = kShortWarps * 256 * 2 * sizeof(C2<float>);
-    static constexpr size_t off_omc = off_om + 32 * sizeof(C2<float>);
-    static constexpr size_t off_w = off_omc + 32 * sizeof(C2<float>);
-    static constexpr size_t bytes = off_w + 256 * sizeof(float);
-};
-
-__global__ void __launch_bounds__(kShortWarps * 32, 1) shortlist_kernel(const Args a)
-{
-    using L = ShortSmem;
-    extern __shared__ __align__(128) unsigned char smem[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    C2<float> *scratch = reinterpret_cast<C2<float> *>(smem + L::off_scratch) + warp * 512;
-    C2<float> *om = reinterpret_cast<C2<float> *>(smem + L::off_om);
-    C2<float> *omc = reinterpret_cast<C2<float> *>(smem + L::off_omc);
-    float *wt = reinterpret_cast<float *>(smem + L::off_w);
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) wt[i] = a.consts->w32[i];
-    for (int i = threadIdx.x; i < 32; i += blockDim.x) {
-        om[i] = {a.consts->om32[2 * i], a.consts->om32[2 * i + 1]};
-        omc[i] = {a.consts->om32[2 * i], -a.consts->om32[2 * i + 1]};
-    }
-    __syncthreads();
-    for (int i = 2 * (blockIdx.x * kShortWarps + warp); i < a.n_order; i += 2 * gridDim.x * kShortWarps) {
-        const bool two = i + 1 < a.n_order;
-        const uint32_t e[2] = {a.order[i], a.order[two ? i + 1 : i]};
-        const bool on[2] = {a.shortlists[a.entries[e[0]].ord].missing <= a.max_missing,
-                            two && a.shortlists[a.entries[e[1]].ord].missing <= a.max_missing};
-        if (!on[0] && !on[1]) continue;
-        if (a.n_restricted != nullptr && lane == 0) atomicAdd(a.n_restricted, (int)on[0] + (int)on[1]);
-        shortlist_stored(a, e, on, scratch, om, omc, wt, lane);
+        // the shortlisted blocks, by pairs of neighbours in the order (a run holds whole pairs)
+        for (long long j = 2ll * taken(&next_pair); j < mine; j = 2ll * taken(&next_pair)) {
+            const long long o = entry(j);
+            if (o >= a.n_order) continue;
+            const bool two = o + 1 < a.n_order;
+            const uint32_t e[2] = {a.order[o], a.order[two ? o + 1 : o]};
+            const bool on[2] = {restricted(e[0]), two && restricted(e[1])};
+            if (!on[0] && !on[1]) continue;
+            if (a.n_restricted != nullptr && lane == 0) atomicAdd(a.n_restricted, (int)on[0] + (int)on[1]);
+            shortlist_stored(a, e, on, scratch, om, omc, wt, lane);
+        }
     }
 }
 
@@ -2501,8 +2477,8 @@ StoredFn stored_fn_of(const int kind, const bool trace)
 }
 StoredFn stored_fn(const rljsde_plan *p, const int kind, const bool trace)
 {
-    if (kind == kFallback)
-        return trace ? stored_kernel<kLayThreeQuarter, kFallback, true> : stored_kernel<kLayThreeQuarter, kFallback, false>;
+    if (kind == kLearned)
+        return trace ? stored_kernel<kLayThreeQuarter, kLearned, true> : stored_kernel<kLayThreeQuarter, kLearned, false>;
     return p->kind == 1 ? stored_fn_of<kLayGeneral>(kind, trace)
            : p->kind == 3 ? stored_fn_of<kLaySingle>(kind, trace) : stored_fn_of<kLayThreeQuarter>(kind, trace);
 }
@@ -2528,7 +2504,7 @@ void stored_shape(const rljsde_plan *p, const int kind, int &warps, int &grid)
     const int most = stored_warps(kind);
     const int per_sm = p->n_order > 0 ? (p->n_order + p->sm_count - 1) / p->sm_count : 1;
     const int rounds = (per_sm + most - 1) / most;
-    warps = kind == kFallback ? most : (per_sm + rounds - 1) / rounds;
+    warps = kind == kLearned ? most : (per_sm + rounds - 1) / rounds;
     const int want = (p->n_order + warps - 1) / warps;
     grid = want < p->sm_count ? (want > 0 ? want : 1) : p->sm_count;
 }
@@ -2845,16 +2821,8 @@ int rljsde_reconstruct_learned(const rljsde_plan_t *plan, const float *lr, size_
     a.n_restricted = n_restricted;
     // shortlist blocks first, then the full loop on the rest
     // with every table set's Gram matrix stored, both loops read its columns
-    if (plan->n_stored > 0 && plan->n_stored == plan->n_tables) {
-        if (cudaFuncSetAttribute(shortlist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ShortSmem::bytes) !=
-            cudaSuccess)
-            return RLJSDE_ERR_CUDA;
-        const int want = (plan->n_order + 2 * kShortWarps - 1) / (2 * kShortWarps);
-        shortlist_kernel<<<want < plan->sm_count ? want : plan->sm_count, kShortWarps * 32, ShortSmem::bytes,
-                           (cudaStream_t)stream>>>(a);
-        if (cudaGetLastError() != cudaSuccess) return RLJSDE_ERR_CUDA;
-        return launch_stored(plan, a, kFallback, (cudaStream_t)stream);
-    }
+    if (plan->n_stored > 0 && plan->n_stored == plan->n_tables)
+        return launch_stored(plan, a, kLearned, (cudaStream_t)stream);
     int st = launch_mode(plan, a, 1, plan->learned_warps, plan->learned_minb, (cudaStream_t)stream);
     if (st == RLJSDE_OK) st = launch_mode(plan, a, 2, 4, 0, (cudaStream_t)stream);
     return st;
