@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(128, 4) conv1_image_kernel(const float *lr, lo
 // 256 positions: 5.5x the multiplications).  Everything is FP32 on the CUDA
 // cores: with the operands in shared memory each kernel below issues three to
 // five FMAs per shared-memory wavefront, so the FMA pipes bound them.  A batch
-// of 4096 patches, loss and gradient: 13.9 -> 0.99 ms against one thread per
+// of 4096 patches, loss and gradient: 13.9 -> 0.71 ms against one thread per
 // output position over the full patches; the sums, split and added in a fixed
 // order, are also closer to the 64-bit gradient (7.6e-7 -> 0.8e-7).
 // A warp owns a sample; its lanes are the 32 channels.
@@ -149,6 +149,26 @@ __global__ void __launch_bounds__(128, 4) conv1_image_kernel(const float *lr, lo
 constexpr int kP1 = 121, kP2 = 25, kP3 = 9;
 constexpr int kZ = 1028;                      // row length of the logits (16-byte rows)
 constexpr int kWRow = 33;                     // weight rows of 32 in shared memory: transposing stores without conflicts
+
+// The 13x13 centre of a patch's five planes, put (ci, y, x, value), nine loads
+// of a lane in flight at a time.
+template <typename Put>
+__device__ __forceinline__ void stage_patch(const float *x, const int lane, Put put)
+{
+    for (int i0 = 0; i0 < 5 * 169; i0 += 9 * 32) {
+        float v[9];
+#pragma unroll
+        for (int j = 0; j < 9; ++j) {
+            const int i = i0 + 32 * j + lane, ci = i / 169, y = (i / 13) % 13, xx = i % 13;
+            v[j] = i < 5 * 169 ? x[ci * 256 + (y + 2) * 16 + xx + 2] : 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < 9; ++j) {
+            const int i = i0 + 32 * j + lane;
+            if (i < 5 * 169) put(i / 169, (i / 13) % 13, i % 13, v[j]);
+        }
+    }
+}
 
 // Forward: x [n][5][16][16] -> a1, a2, f.  Same order of additions per output
 // as a direct loop over input channels and taps.
@@ -176,16 +196,14 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 1) train_fwd_kernel(const floa
         const int2 blk = blocks[s];
         const int oy = 2 * blk.x - 8, ox = 2 * blk.y - 8;              // the patch's first L-pixel (even)
         __syncwarp();
-        for (int i = lane; i < 5 * 13 * 13; i += 32) {
-            const int ci = i / 169, y = (i / 13) % 13, xx = i % 13;
-            X[(ci * 13 + y) * 16 + xx] = x[((size_t)s * 5 + ci) * 256 + (y + 2) * 16 + xx + 2];
-        }
+        stage_patch(x + (size_t)s * 5 * 256, lane, [&](int ci, int y, int xx, float v) { X[(ci * 13 + y) * 16 + xx] = v; });
         __syncwarp();
         // conv1, one output row at a time
         for (int ry = 0; ry < 11; ++ry) {
             float acc[11];
 #pragma unroll
             for (int c = 0; c < 11; ++c) acc[c] = b1;
+#pragma unroll
             for (int ci = 0; ci < 5; ++ci)
 #pragma unroll
                 for (int dy = 0; dy < 3; ++dy) {
@@ -314,20 +332,28 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 1) train_bwd_kernel(const floa
     __syncthreads();
     for (int s = blockIdx.x * kBwdWarps + warp; s < n; s += gridDim.x * kBwdWarps) {
         __syncwarp();
+        {
+            // (all loads before the first store: the compiler keeps their order)
+            float v[9], fv[9];
+            const size_t i = (size_t)s * kHeadIn + lane * 9;
 #pragma unroll
-        for (int t = 0; t < 9; ++t) {
-            const size_t i = (size_t)s * kHeadIn + lane * 9 + t;
-            float v = gf[i];
-            for (int p = 1; p < parts; ++p) v += gf[(size_t)p * n * kHeadIn + i];
-            v = f[i] > 0.f ? v : 0.f;
-            g3[((size_t)s * kP3 + t) * kC + lane] = v;
-            G3[lane * 12 + (t / 3) * 4 + t % 3] = v;
+            for (int t = 0; t < 9; ++t) { v[t] = gf[i + t]; fv[t] = f[i + t]; }
+            for (int p = 1; p < parts; ++p)
+#pragma unroll
+                for (int t = 0; t < 9; ++t) v[t] += gf[(size_t)p * n * kHeadIn + i + t];
+#pragma unroll
+            for (int t = 0; t < 9; ++t) {
+                v[t] = fv[t] > 0.f ? v[t] : 0.f;
+                g3[((size_t)s * kP3 + t) * kC + lane] = v[t];
+                G3[lane * 12 + (t / 3) * 4 + t % 3] = v[t];
+            }
         }
         __syncwarp();
         {
-            float acc[25];
+            float acc[25], av[25];
+            const size_t i = (size_t)s * kP2 * kC + lane;
 #pragma unroll
-            for (int p = 0; p < 25; ++p) acc[p] = 0.f;
+            for (int p = 0; p < 25; ++p) { acc[p] = 0.f; av[p] = a2[i + p * kC]; }
 #pragma unroll 2
             for (int co = 0; co < kC; ++co) {
                 float w[9];
@@ -345,9 +371,8 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 1) train_bwd_kernel(const floa
             }
 #pragma unroll
             for (int p = 0; p < 25; ++p) {
-                const size_t i = ((size_t)s * kP2 + p) * kC + lane;
-                const float v = a2[i] > 0.f ? acc[p] : 0.f;
-                g2[i] = v;
+                const float v = av[p] > 0.f ? acc[p] : 0.f;
+                g2[i + p * kC] = v;
                 G2[lane * 40 + (p / 5) * 8 + p % 5] = v;
             }
         }
@@ -371,8 +396,19 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 1) train_bwd_kernel(const floa
             }
         }
         const size_t base = (size_t)s * kP1 * kC + lane;
+        // a row's loads before its stores, the next row's in flight meanwhile
+        float av[2][11];
 #pragma unroll
-        for (int p = 0; p < kP1; ++p) g1[base + p * kC] = a1[base + p * kC] > 0.f ? acc[p] : 0.f;
+        for (int c = 0; c < 11; ++c) av[0][c] = a1[base + c * kC];
+#pragma unroll
+        for (int ry = 0; ry < 11; ++ry) {
+            if (ry < 10) {
+#pragma unroll
+                for (int c = 0; c < 11; ++c) av[(ry + 1) & 1][c] = a1[base + ((ry + 1) * 11 + c) * kC];
+            }
+#pragma unroll
+            for (int c = 0; c < 11; ++c) g1[base + (ry * 11 + c) * kC] = av[ry & 1][c] > 0.f ? acc[ry * 11 + c] : 0.f;
+        }
     }
 }
 
@@ -392,13 +428,30 @@ __global__ void __launch_bounds__(256, 2) train_dw_kernel(const float *g, const 
     for (int c = 0; c < 4; ++c)
 #pragma unroll
         for (int t = 0; t < 9; ++t) acc[c][t] = 0.f;
+    // the next sample's operands are fetched into registers while this one's are used
+    constexpr int NAV = (HI * HI * kC / 4 + 255) / 256, NGV = (HO * HO * kC / 4 + 255) / 256;
+    float4 ra[NAV], rg[NGV];
+    auto fetch = [&](const int s) {
+        const float4 *pa = reinterpret_cast<const float4 *>(a + (size_t)s * HI * HI * kC);
+        const float4 *pg = reinterpret_cast<const float4 *>(g + (size_t)s * HO * HO * kC);
+#pragma unroll
+        for (int j = 0; j < NAV; ++j)
+            if (threadIdx.x + 256 * j < HI * HI * kC / 4) ra[j] = pa[threadIdx.x + 256 * j];
+#pragma unroll
+        for (int j = 0; j < NGV; ++j)
+            if (threadIdx.x + 256 * j < HO * HO * kC / 4) rg[j] = pg[threadIdx.x + 256 * j];
+    };
+    if (blockIdx.x < n) fetch(blockIdx.x);
     for (int s = blockIdx.x; s < n; s += gridDim.x) {
         __syncthreads();
-        const float4 *src = reinterpret_cast<const float4 *>(a + (size_t)s * HI * HI * kC);
-        for (int i = threadIdx.x; i < HI * HI * kC / 4; i += 256) reinterpret_cast<float4 *>(as)[i] = src[i];
-        src = reinterpret_cast<const float4 *>(g + (size_t)s * HO * HO * kC);
-        for (int i = threadIdx.x; i < HO * HO * kC / 4; i += 256) reinterpret_cast<float4 *>(gs)[i] = src[i];
+#pragma unroll
+        for (int j = 0; j < NAV; ++j)
+            if (threadIdx.x + 256 * j < HI * HI * kC / 4) reinterpret_cast<float4 *>(as)[threadIdx.x + 256 * j] = ra[j];
+#pragma unroll
+        for (int j = 0; j < NGV; ++j)
+            if (threadIdx.x + 256 * j < HO * HO * kC / 4) reinterpret_cast<float4 *>(gs)[threadIdx.x + 256 * j] = rg[j];
         __syncthreads();
+        if (s + (int)gridDim.x < n) fetch(s + gridDim.x);
 #pragma unroll 1
         for (int ho = 0; ho < HO; ++ho) {
             float4 q[HO];
@@ -451,17 +504,21 @@ __global__ void __launch_bounds__(kDw1Warps * 32, 2) train_dw1_kernel(const floa
     for (int s = blockIdx.x * kDw1Warps + warp; s < n; s += gridDim.x * kDw1Warps) {
         float *X = xs[warp];
         __syncwarp();
-        for (int i = lane; i < 5 * 169; i += 32) {
-            const int ci = i / 169, y = (i / 13) % 13, xx = i % 13;
-            X[(y * 13 + xx) * 8 + ci] = x[((size_t)s * 5 + ci) * 256 + (y + 2) * 16 + xx + 2];
-        }
+        stage_patch(x + (size_t)s * 5 * 256, lane, [&](int ci, int y, int xx, float v) { X[(y * 13 + xx) * 8 + ci] = v; });
         __syncwarp();
         const float *g = g1 + (size_t)s * kP1 * kC + lane;
+        float gn[11];                                                  // the next row's gradients, in flight
+#pragma unroll
+        for (int c = 0; c < 11; ++c) gn[c] = g[c * kC];
 #pragma unroll 1
         for (int ry = 0; ry < 11; ++ry) {
             float gv[11];
 #pragma unroll
-            for (int c = 0; c < 11; ++c) gv[c] = g[(ry * 11 + c) * kC];
+            for (int c = 0; c < 11; ++c) gv[c] = gn[c];
+            if (ry < 10) {
+#pragma unroll
+                for (int c = 0; c < 11; ++c) gn[c] = g[((ry + 1) * 11 + c) * kC];
+            }
             float v[3][3][5];                                          // [column mod 3][row][ci]
 #pragma unroll
             for (int col = 0; col < 13; ++col) {
@@ -499,24 +556,58 @@ __global__ void __launch_bounds__(kDw1Warps * 32, 2) train_dw1_kernel(const floa
     }
 }
 
-// out[i] = sum of parts[p][i], p < np, for a segment of `len` values: eight
-// warps of a CTA take every eighth part for 32 values, then add up in order.
-__global__ void __launch_bounds__(256) sum_parts_kernel(const float *parts, int np, int len, float *out)
+// Every partial gradient of a step in one launch.  Segment: out[i] = sum of
+// parts[p][i], p < np, for len values; eight warps of a CTA take every eighth
+// part for 32 values, then add up in order.  The last CTA averages the
+// samples' losses.
+struct SumSegment {
+    const float *parts;
+    float *out;
+    int np, len, first;                   // first: the segment's first CTA
+};
+constexpr int kSegments = 5;
+struct SumArgs {
+    SumSegment seg[kSegments];
+    int ctas;                             // of all segments; one more for the loss
+    const float *loss;
+    int n;
+    float *mean;
+};
+
+__global__ void __launch_bounds__(256) sum_parts_kernel(const SumArgs a)
 {
+    if ((int)blockIdx.x == a.ctas) {
+        __shared__ double acc[256];
+        double v = 0.0;
+        for (int i = threadIdx.x; i < a.n; i += 256) v += a.loss[i];
+        acc[threadIdx.x] = v;
+        __syncthreads();
+        for (int o = 128; o > 0; o >>= 1) {
+            if (threadIdx.x < o) acc[threadIdx.x] += acc[threadIdx.x + o];
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) *a.mean = (float)(acc[0] / a.n);
+        return;
+    }
     __shared__ float red[8][32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+    int j = 0;
+#pragma unroll
+    for (int q = 1; q < kSegments; ++q)
+        if ((int)blockIdx.x >= a.seg[q].first) j = q;
+    const SumSegment seg = a.seg[j];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = ((int)blockIdx.x - seg.first) * 32 + lane;
     float v = 0.f;
-    if (i < len) {
+    if (i < seg.len) {
 #pragma unroll 4
-        for (int p = warp; p < np; p += 8) v += parts[(size_t)p * len + i];
+        for (int p = warp; p < seg.np; p += 8) v += seg.parts[(size_t)p * seg.len + i];
     }
     red[warp][lane] = v;
     __syncthreads();
-    if (warp == 0 && i < len) {
+    if (warp == 0 && i < seg.len) {
         v = red[0][lane];
 #pragma unroll
         for (int w = 1; w < 8; ++w) v += red[w][lane];
-        out[i] = v;
+        seg.out[i] = v;
     }
 }
 
@@ -679,13 +770,19 @@ __global__ void __launch_bounds__(256) loss_kernel(float *z, const float *bias, 
     if (s >= n) return;
     float *zs = z + (size_t)s * kZ;
     float l = 0.f;
-    uint32_t key[32];
+    uint32_t key[32], ts = 0;                 // (loads before the stores to z: the compiler keeps their order)
 #pragma unroll
     for (int j = 0; j < 32; ++j) {
         const int k = lane + 32 * j;
-        const float zk = zs[k] + bias[k];
-        key[j] = order_key(zk);
-        const float tk = t[(size_t)s * 1024 + k] ? 1.f : 0.f;
+        key[j] = order_key(zs[k] + bias[k]);
+        ts |= (t[(size_t)s * 1024 + k] ? 1u : 0u) << j;
+    }
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+        const int k = lane + 32 * j;
+        // the logit back from its order key
+        const float zk = __uint_as_float(key[j] ^ (((key[j] >> 31) - 1u) | 0x80000000u));
+        const float tk = (ts >> j) & 1u ? 1.f : 0.f;
         const float w = tk > 0.5f ? pos_w : 1.f;
         const float sp = fmaxf(zk, 0.f) + log1pf(expf(-fabsf(zk)));
         l += w * (sp - tk * zk) / 1024.f;
@@ -732,21 +829,6 @@ __global__ void __launch_bounds__(256) loss_kernel(float *z, const float *bias, 
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
     if (lane == 0) loss[s] = l;
-}
-
-// *out = sum of the samples' losses / n, in a fixed order.
-__global__ void __launch_bounds__(256) mean_kernel(const float *v, int n, float *out)
-{
-    __shared__ double red[256];
-    double a = 0.0;
-    for (int i = threadIdx.x; i < n; i += 256) a += v[i];
-    red[threadIdx.x] = a;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *out = (float)(red[0] / n);
 }
 
 __global__ void adam_kernel(float *p, const float *g, float *m, float *v, int n, float lr, float b1, float b2,
@@ -1685,8 +1767,8 @@ namespace {
 constexpr int kDwhParts = 12;                 // 27 tiles each: 324 CTAs, about two per SM
 constexpr int kGfParts = 3;
 constexpr size_t kDwhFloats = (size_t)kOut * kHeadIn;
-constexpr int kMaxSms = 512;                  // most SMs a device is taken to have: rows of conv partial gradients
-constexpr size_t kPartFloats = kDwhParts * (kDwhFloats + kOut) + 2 * (size_t)kMaxSms * kDwPart;
+constexpr int kConvParts = 400;               // most partial gradients of a convolution
+constexpr size_t kPartFloats = kDwhParts * (kDwhFloats + kOut) + (size_t)kConvParts * (2 * kDwPart + kDw1Part);
 
 void free_train(rljsde_net *n)
 {
@@ -1774,13 +1856,11 @@ void refresh_bf16(rljsde_net *n, cudaStream_t s)
                                                                              n->conv_packed + tc::kBBytes);
 }
 
-int sms_of(const rljsde_net *net) { return net->sm_count < kMaxSms ? net->sm_count : kMaxSms; }
-
 // Forward over n patches: a1, a2, f and the head logits (without bias) in z.
 int forward_patches(rljsde_net *net, const float *x, const int32_t *blocks, int n, int lr_h, int lr_w, cudaStream_t s)
 {
     const float *r = net->rounded, *b = net->master;     // weights bf16-rounded, biases FP32
-    const int sms = sms_of(net);
+    const int sms = net->sm_count;
     if (cudaFuncSetAttribute(train_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFwdSmem) != cudaSuccess)
         return RLJSDE_ERR_CUDA;
     const int g = (n + kFwdWarps - 1) / kFwdWarps;
@@ -1945,18 +2025,16 @@ static int loss_grad(rljsde_net *net, const float *x, const int32_t *blocks, int
     st = forward_patches(net, x, blocks, n, lr_h, lr_w, s);
     if (st) return st;
     const float *r = net->rounded;
-    const int sms = sms_of(net);
+    const int sms = net->sm_count;
     loss_kernel<<<(n + 7) / 8, 256, 0, s>>>(net->z, net->master + kBh, targets, nu_t, mass, n, pos_w, nu_w, gate_w,
                                             net->loss + 4);
-    mean_kernel<<<1, 256, 0, s>>>(net->loss + 4, n, net->loss);
     // head: gWh[k][j] = sum_s gz[s][k] f[s][j], gbh[k] = sum_s gz[s][k]; gf[s][j] = sum_k gz[s][k] Wh[k][j]
     const int want = (n + 127) / 128, parts = want < kDwhParts ? want : kDwhParts;
     const int kpart = ((n + parts - 1) / parts + 15) / 16 * 16, np = (n + kpart - 1) / kpart;
-    float *dwh = net->part, *dbh = dwh + kDwhParts * kDwhFloats, *dw = dbh + (size_t)kDwhParts * kOut;
+    float *dwh = net->part, *dbh = dwh + kDwhParts * kDwhFloats, *dw3 = dbh + (size_t)kDwhParts * kOut,
+          *dw2 = dw3 + (size_t)kConvParts * kDwPart, *dw1 = dw2 + (size_t)kConvParts * kDwPart;
     head_gemm_kernel<8, 6, false, false, true><<<dim3(3, 9, np), 256, 0, s>>>(
         kOut, kHeadIn, n, kpart, net->z, kZ, net->f, kHeadIn, dwh, kHeadIn, (long long)kDwhFloats, dbh);
-    sum_parts_kernel<<<(int)(kDwhFloats + 31) / 32, 256, 0, s>>>(dwh, np, (int)kDwhFloats, net->grad + kWh);
-    sum_parts_kernel<<<(kOut + 31) / 32, 256, 0, s>>>(dbh, np, kOut, net->grad + kBh);
     const int gfk = (kOut / kGfParts + 15) / 16 * 16;                  // 352, 352, 322
     if ((n + 127) / 128 * 9 >= sms)
         head_gemm_kernel<8, 6, true, false, false><<<dim3(3, (n + 127) / 128, kGfParts), 256, 0, s>>>(
@@ -1969,15 +2047,23 @@ static int loss_grad(rljsde_net *net, const float *x, const int32_t *blocks, int
     const int gb = (n + kBwdWarps - 1) / kBwdWarps;
     train_bwd_kernel<<<gb < sms ? gb : sms, kBwdWarps * 32, kBwdSmem, s>>>(net->gf, kGfParts, r, n, net->a1, net->a2, net->f,
                                                                         net->g1, net->g2, net->g3);
-    // conv weight gradients: per-CTA partial sums, then their sum (weights and bias are adjacent in grad)
-    const int gd = n < 2 * sms ? n : 2 * sms;
-    train_dw_kernel<3, 5, 1><<<gd, 256, 0, s>>>(net->g3, net->a2, n, dw);
-    sum_parts_kernel<<<(kDwPart + 31) / 32, 256, 0, s>>>(dw, gd, kDwPart, net->grad + kW3);
-    train_dw_kernel<5, 11, 2><<<gd, 256, 0, s>>>(net->g2, net->a1, n, dw);
-    sum_parts_kernel<<<(kDwPart + 31) / 32, 256, 0, s>>>(dw, gd, kDwPart, net->grad + kW2);
-    const int g1 = (n + kDw1Warps - 1) / kDw1Warps, gd1 = g1 < 2 * sms ? g1 : 2 * sms;
-    train_dw1_kernel<<<gd1, kDw1Warps * 32, 0, s>>>(net->g1, x, n, dw);
-    sum_parts_kernel<<<(kDw1Part + 31) / 32, 256, 0, s>>>(dw, gd1, kDw1Part, net->grad + kW1);
+    // conv weight gradients: per-CTA partial sums, then all sums (weights and bias are adjacent in grad)
+    const int most = 2 * sms < kConvParts ? 2 * sms : kConvParts;
+    const int gd = n < most ? n : most, g1 = (n + kDw1Warps - 1) / kDw1Warps, gd1 = g1 < most ? g1 : most;
+    train_dw_kernel<3, 5, 1><<<gd, 256, 0, s>>>(net->g3, net->a2, n, dw3);
+    train_dw_kernel<5, 11, 2><<<gd, 256, 0, s>>>(net->g2, net->a1, n, dw2);
+    train_dw1_kernel<<<gd1, kDw1Warps * 32, 0, s>>>(net->g1, x, n, dw1);
+    SumArgs sa{{{dwh, net->grad + kWh, np, (int)kDwhFloats, 0},
+                {dbh, net->grad + kBh, np, kOut, 0},
+                {dw3, net->grad + kW3, gd, kDwPart, 0},
+                {dw2, net->grad + kW2, gd, kDwPart, 0},
+                {dw1, net->grad + kW1, gd1, kDw1Part, 0}},
+               0, net->loss + 4, n, net->loss};
+    for (auto &seg : sa.seg) {
+        seg.first = sa.ctas;
+        sa.ctas += (seg.len + 31) / 32;
+    }
+    sum_parts_kernel<<<sa.ctas + 1, 256, 0, s>>>(sa);
     if (cudaGetLastError() != cudaSuccess) return RLJSDE_ERR_CUDA;
     if (loss_host && cudaMemcpyAsync(loss_host, net->loss, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess)
         return RLJSDE_ERR_CUDA;
