@@ -129,8 +129,8 @@ typedef struct {
                              the stored-C loop runs one CTA of up to 12 warps per
                              SM, a block per warp (rljsde_set_launch and
                              rljsde_autotune shape the factored loop).  The
-                             learned proposal's loops always use the factored
-                             form                                              */
+                             learned proposal's loops read the stored matrices
+                             when every table set has one                      */
 } rljsde_params;
 
 /* Fill *p with the defaults above.  Returns RLJSDE_ERR_INVALID_ARG on NULL. */

@@ -14,18 +14,18 @@
 //        - read from the Gram matrix the plan stores for the block's local
 //          mask (the paper's recurrent form, Table I; the default), the state
 //          kept as sqrt(q_k / D_k) R_k so that the score is its squared
-//          modulus (greedy_loop_stored), or
+//          modulus (stored_kernel; FP64 plans keep R: stored64_kernel), or
 //        - rebuilt from the factored tables, the update carried out on Y:
 //            Y_t(kap) -= gamma delta h_t(uv) G_t((uv - kap) mod 16),
 //          which is Eq. 17 with C factored as C_{k,l} = sum_t conj(h_t(k))
-//          h_t(l) G_t(l - k) (greedy_loop_f32, and the FP64 loop);
+//          h_t(l) G_t(l - k) (greedy_loop_f32, and greedy_loop for FP64);
 //   4. Eq. 18 on the central block, accumulated as each coefficient changes.
-// A persistent CTA walks chunks of 8 blocks that share one table set; the
-// table set of the next chunk of the same slot parity is brought into shared
-// memory with a bulk asynchronous copy (cp.async.bulk + mbarrier) while the
-// current chunk runs.
+// In the factored kernels a persistent CTA walks chunks of 8 blocks that share
+// one table set; the table set of the next chunk of the same slot parity is
+// brought into shared memory with a bulk asynchronous copy (cp.async.bulk +
+// mbarrier) while the current chunk runs.
 //
-// Direct path (Sec. IV, Eqs. 4-10): one warp per block keeps the residual r
+// Direct path (Sec. IV, Eqs. 4-10): one CTA per block keeps the residual r
 // and recomputes the O(W^4) projection of Eq. 10 every iteration.
 #include <cuda_runtime.h>
 
@@ -138,7 +138,7 @@ struct Args {
     const int *cslot;                      // per table set: its stored matrix, or -1 (factored)
     int cfilter;                           // chunks a factored launch takes: 0 all, 1 those whose table
                                            // set has no stored matrix
-    const unsigned char *cstore64;         // the same for FP64 plans, kStored64Bytes each
+    const unsigned char *cstore64;         // the same memory by bytes (FP64 plans: kStored64Bytes each)
     const uint32_t *order;                 // stored-C loop: the entries of the stored table sets
     int n_order;
     const Consts *consts;
