@@ -1153,12 +1153,11 @@ __device__ __forceinline__ void stored_block_pairs(const Args &a, const float4 *
         r_at_slot(R, bk >> 5, mre, mim);
         const float Rre = __shfl_sync(0xffffffffu, mre, lane_of(bk));
         const float Rim = __shfl_sync(0xffffffffu, mim, lane_of(bk));
-        int u, v;
-        C2<float> g[4];
+        const int u = bk >> 5, v = bk & 31;
         const C2<float> gd = {gamma * (Rre * invD), gamma * (Rim * invD)};   // as in select_step
-        Args quiet = a;
-        quiet.trace_sel = nullptr;
-        select_step<float, LAY, true>(quiet, om, invD, gamma, bk, Rre, Rim, eta, gam, lane, 0, it, u, v, g, fpix, pw);
+        const C2<float> ph = om[(eta * u + gam * v) & 31];
+        pw = ((u & 15) == 0 && (v & 15) == 0) ? 0.f : 1.f;
+        fpix += (1.f + pw) * (gd.re * ph.re - gd.im * ph.im);
         if constexpr (TRACE) {
             if (lane == 0) {
                 const long long row = (long long)we.ord * a.nu_max + it;
