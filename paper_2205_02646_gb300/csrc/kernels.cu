@@ -29,6 +29,7 @@
 // and recomputes the O(W^4) projection of Eq. 10 every iteration.
 #include <cuda_runtime.h>
 
+#include <climits>
 #include <cstdint>
 
 #include "rljsde_internal.h"
@@ -1907,15 +1908,25 @@ __global__ void __launch_bounds__(stored_warps(KIND) * 32, 1) stored_kernel(cons
 // the FP32 rate, so nothing else matters: the scores are screened in FP32 from
 // the top bits of R (integer operations; an FP64-to-FP32 conversion would cost
 // as much as a multiply-add) and only candidates within 2^-18 of the largest
-// screened score get their FP64 score, rounded to binary32 as before.  The
-// screen's relative error is below 2^-20: R's components are truncated to 24
-// bits (2^-23), q / D and the four operations round at 2^-24 each.
+// screened score get their FP64 score, rounded to binary32 as before.
+// The screened score is q' |x|^2, q / D = 4^E q' with E such that the table
+// set's largest q' is just below 1, x = 2^-T R with T such that the largest
+// score of the iteration before is about 1.  It serves where its largest value M
+// is at least 2^-60 and every component of x below 2^32: a score near M then
+// has q' above 2^-126 and a component above 2^-32, and is off by relative steps
+// only, the components truncated to 24 bits (2^-23, squared 2^-22), q' and three
+// operations rounded at 2^-24 each, 2^-21 in all, while two scores equal in
+// binary32 are 2^-23 apart; and a q' below 2^-126, taken as 0, stays below M / 2.
+// Elsewhere, and where the scores leave binary32's normal range (they then tie,
+// or all are 0), or E is beyond 300 (products that leave FP64's own range),
+// every candidate is scored in FP64.
 //
 // Lane (kap2 = lane & 15, h = lane >> 4) holds slots s = 16 a + 2 i + b, k =
 // (8 h + i + 16 a, kap2 + 16 b): increasing k, the initial projection's layout.
 // Table set: 1024 columns of [slot][lane] (re, im); q / D then 1 / D by k in
-// FP64; q / D rounded to FP32 as [slot][lane].
-// 256x256, nu_max 100: 21.3 -> 3.6 ms, 151 FP64 instructions an iteration (FP64 floor 2.0 ms).
+// FP64; q' as floats by [slot][lane]; E.
+// 256x256, nu_max 100: 21.3 -> 3.65 ms, 151 FP64 instructions an iteration (at 16
+// cycles each 3.15 ms; the update alone, 128 of them, 2.67 ms).
 __host__ __device__ constexpr int slot64_k(int s, int lane)
 {
     return (8 * (lane >> 4) + ((s >> 1) & 7) + 16 * (s >> 4)) * kW + (lane & 15) + 16 * (s & 1);
@@ -1931,15 +1942,16 @@ struct Stored64Smem {
     static constexpr size_t bytes = off_w + 256 * sizeof(double);
 };
 
-// |x| truncated to 24 significant bits as a float (0 below 2^-127; the
-// caller looks at `top`, the largest biased-down exponent word, for values a
-// float does not hold).
-__device__ __forceinline__ float screen(const double x, int &top)
+// |x| scaled by the power of two that `shift` adds to its upper word (which
+// takes the float's bias for the double's too), truncated to 24 significant
+// bits as a float, 0 below 2^-126; top: the largest upper word so far.
+__device__ __forceinline__ float screen(const double x, const int shift, int &top)
 {
-    const int e = max((__double2hiint(x) & 0x7fffffff) - (896 << 20), 0);
+    const int e = max((__double2hiint(x) & 0x7fffffff) + shift, 0);
     top = max(top, e);
     return __uint_as_float(__funnelshift_l((unsigned)__double2loint(x), (unsigned)e, 3));
 }
+constexpr int kScreenMaxE = 300, kScreenMaxT = 50;      // |E|; |E + T|, half the exponent of binary32's normal range
 
 template <int LAY>
 __global__ void __launch_bounds__(kStored64Warps * 32, 1) stored64_kernel(const Args a)
@@ -1966,6 +1978,7 @@ __global__ void __launch_bounds__(kStored64Warps * 32, 1) stored64_kernel(const 
         const unsigned char *tab = a.cstore64 + (size_t)a.cslot[t] * kStored64Bytes;
         const double *qd = reinterpret_cast<const double *>(tab + kStored64ColsBytes), *invd = qd + kK;
         const float *qf = reinterpret_cast<const float *>(invd + kK) + lane;
+        const int E = *reinterpret_cast<const int *>(qf - lane + kK);
         C2<double> R[32];
         {
             const uint8_t *types = a.records + (size_t)t * sizeof(Record<double>) + offsetof(Record<double>, types);
@@ -1980,19 +1993,22 @@ __global__ void __launch_bounds__(kStored64Warps * 32, 1) stored64_kernel(const 
             }
         }
         double fpix = 0;
+        int T = -E;
         const long long trow = (long long)we.ord * a.nu_max;
         for (int it = 0;;) {
             float s32[32], m = 0.f;
             int top = 0;
+            const int shift = (127 - 1023 - T) * (1 << 20);
 #pragma unroll
             for (int s = 0; s < 32; ++s) {
-                const float re = screen(R[s].re, top), im = screen(R[s].im, top);
+                const float re = screen(R[s].re, shift, top), im = screen(R[s].im, shift, top);
                 s32[s] = ldg_stream1(qf + 32 * s) * fmaf(re, re, im * im);
                 m = fmaxf(m, s32[s]);
             }
             const float M = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));
-            // outside the floats' safe range every candidate gets its FP64 score
-            const bool every = __any_sync(0xffffffffu, top >= ((127 + 60) << 20)) || !(M >= 0x1p-100f && M <= 0x1p+100f);
+            const int lg = (int)(__float_as_uint(M) >> 23) - 127;         // M's exponent; lg + 2 (E + T) the score's
+            const bool every = __any_sync(0xffffffffu, top >= ((127 + 32) << 20)) || lg < -60 || abs(E) > kScreenMaxE ||
+                               abs(lg + 2 * (E + T)) > 2 * kScreenMaxT;
             const float least = every ? -1.f : M * (1.f - 0x1p-18f);
             // slots any lane has to look at: a branch over each of the others
             // (predicated, their FP64 instructions would still take the pipe)
@@ -2002,7 +2018,7 @@ __global__ void __launch_bounds__(kStored64Warps * 32, 1) stored64_kernel(const 
                 if (every || s32[s] >= least) hits |= 1u << s;
             const unsigned any = __reduce_or_sync(0xffffffffu, hits);
             unsigned bits = 0;                            // binary32 score + 1, 0 = none
-            int bk = kK - 1;
+            int bk = 0;
             double bre = 0, bim = 0;
 #pragma unroll
             for (int s = 0; s < 32; ++s)
@@ -2010,12 +2026,14 @@ __global__ void __launch_bounds__(kStored64Warps * 32, 1) stored64_kernel(const 
                     asm volatile("" ::: "memory");
                     const int k = slot64_k(s, lane);
                     const float key = (float)(qd[k] * (R[s].re * R[s].re + R[s].im * R[s].im));
-                    if (((hits >> s) & 1u) && __float_as_uint(key) + 1 > bits) {
+                    // (key is NaN where q / D is infinite and R zero: no candidate)
+                    if (((hits >> s) & 1u) && key >= 0.f && __float_as_uint(key) + 1 > bits) {
                         bits = __float_as_uint(key) + 1; bk = k; bre = R[s].re; bim = R[s].im;
                     }
                 }
             const unsigned most = __reduce_max_sync(0xffffffffu, bits);
             bk = (int)__reduce_min_sync(0xffffffffu, bits == most ? (unsigned)bk : (unsigned)(kK - 1));
+            T = min(max(((int)((most - 1) >> 23) - 127) >> 1, -kScreenMaxT), kScreenMaxT) - E;
             const int wl = (bk & 15) + ((bk >> 5) & 8) * 2;
             const double Rre = __shfl_sync(0xffffffffu, bre, wl), Rim = __shfl_sync(0xffffffffu, bim, wl);
             const double invD = invd[bk];
@@ -2668,14 +2686,25 @@ __global__ void __launch_bounds__(512) build_c_kernel(const double *g64, const C
     }
 }
 
-// q / D and 1 / D of an FP64 table set (see stored64_kernel).
+// q / D and 1 / D of an FP64 table set, and its q' and E (see stored64_kernel).
 __global__ void __launch_bounds__(512) build_c64_tables_kernel(const double *g64, unsigned char *out)
 {
     const double *src = g64 + (size_t)blockIdx.x * kStoredBuildDoubles + 2048;
     double *d = reinterpret_cast<double *>(out + (size_t)blockIdx.x * kStored64Bytes + kStored64ColsBytes);
     float *qf = reinterpret_cast<float *>(d + 2 * kK);
     for (int i = threadIdx.x; i < 2 * kK; i += blockDim.x) d[i] = src[i];
-    for (int i = threadIdx.x; i < kK; i += blockDim.x) qf[i] = (float)src[slot64_k(i >> 5, i & 31)];
+    // E of the largest q / D, from its upper word (0 where all are 0; an infinite one has E = 513)
+    __shared__ int most;
+    if (threadIdx.x == 0) most = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < kK; i += blockDim.x) atomicMax(&most, __double2hiint(src[i]));
+    __syncthreads();
+    const int E = most == 0 ? 0 : (((most >> 20) - 1023) >> 1) + 1;
+    for (int i = threadIdx.x; i < kK; i += blockDim.x) {
+        const float q = (float)scalbn(src[slot64_k(i >> 5, i & 31)], -2 * E);
+        qf[i] = q >= 0x1p-126f ? q : 0.f;
+    }
+    if (threadIdx.x == 0) *reinterpret_cast<int *>(qf + kK) = E;
 }
 
 // The row scales s_k in the lane order and 1 / (s_l D_l) of each stored

@@ -125,9 +125,10 @@ constexpr size_t kStoredTableBytes = kStoredColsBytes + 8192 + 4096;
 constexpr size_t kStoredScaleOff = kStoredColsBytes / 16;          // in float4
 constexpr size_t kStoredInvDOff = kStoredColsBytes / 16 + 512;     // in float4
 // The same of an FP64 plan (auto only): 1024 columns of 1024 (re, im), then
-// q_k / D_k and 1 / D_k by k, then q_k / D_k in FP32 (layout: stored64_kernel).
+// q_k / D_k and 1 / D_k by k, then q_k / D_k scaled into FP32 and the scale
+// (layout: stored64_kernel).
 constexpr size_t kStored64ColsBytes = (size_t)kK * kK * 16;
-constexpr size_t kStored64Bytes = kStored64ColsBytes + kK * (8 + 8 + 4);
+constexpr size_t kStored64Bytes = kStored64ColsBytes + kK * (8 + 8 + 4) + 16;
 // c_supply 3 stores the matrix of a table set that at least this many blocks
 // use (border table sets of a recurrent mask are used by few blocks each);
 // the others run the factored loop in a second kernel.
