@@ -142,6 +142,7 @@ struct Args {
     const unsigned char *cstore64;         // the same memory by bytes (FP64 plans: kStored64Bytes each)
     const uint32_t *order;                 // stored-C loop: the entries of the stored table sets
     int n_order;
+    int run_log;                           // learned path: a CTA takes every gridDim.x-th run of 1 << run_log entries
     const Consts *consts;
     ImageDesc single;          // used when descs == nullptr
     const ImageDesc *descs;
@@ -1789,7 +1790,8 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) recurrent_kernel(const Args 
 // kLearned runs the learned path: the CTA lists its blocks the gate sends
 // back, a batch of its entries at a time, its warps take them from the list,
 // and a warp that finds the list empty goes on to the CTA's shortlisted
-// blocks, two at a time (in two kernels, one after the other, the full loop
+// blocks, two at a time, or singly where the image has no more than a block for
+// each warp (in two kernels, one after the other, the full loop
 // had the SMs to itself while its last blocks ran: 1024x1024, nu_max 100,
 // a tenth of the blocks sent back: 1.72 -> 1.59 ms; 256x256: 381 -> 253 us).
 constexpr int kStoredWarps = 12;
@@ -1862,11 +1864,12 @@ __global__ void __launch_bounds__(stored_warps(KIND) * 32, 1) stored_kernel(cons
     } else {
         __shared__ uint32_t list[kStoredBatch];
         __shared__ int n_list, next, next_pair;
-        // entries o of this CTA: runs of kChunk, every gridDim-th run
-        const long long runs = ((long long)a.n_order + kChunk - 1) / kChunk;
-        const long long mine = ((runs - blockIdx.x + gridDim.x - 1) / gridDim.x) * kChunk;
+        // entries o of this CTA: every gridDim-th run
+        const int rl = a.run_log, step = rl > 0 ? 2 : 1;   // shortlisted blocks a warp takes at a time
+        const long long runs = ((long long)a.n_order + (1 << rl) - 1) >> rl;
+        const long long mine = ((runs - blockIdx.x + gridDim.x - 1) / gridDim.x) << rl;
         auto entry = [&](const long long j) {             // this CTA's j-th place in the order, or beyond its end
-            return ((j / kChunk) * gridDim.x + blockIdx.x) * kChunk + j % kChunk;
+            return (((j >> rl) * gridDim.x + blockIdx.x) << rl) + (j & ((1 << rl) - 1));
         };
         auto taken = [&](int *counter) {                  // the next number for this warp
             int i = 0;
@@ -1886,11 +1889,11 @@ __global__ void __launch_bounds__(stored_warps(KIND) * 32, 1) stored_kernel(cons
             __syncthreads();
             for (int i = taken(&next); i < n_list; i = taken(&next)) block(list[i]);
         }
-        // the shortlisted blocks, by pairs of neighbours in the order (a run holds whole pairs)
-        for (long long j = 2ll * taken(&next_pair); j < mine; j = 2ll * taken(&next_pair)) {
+        // the shortlisted blocks, by pairs of neighbours in the order (a run holds whole pairs), or singly
+        for (long long j = (long long)step * taken(&next_pair); j < mine; j = (long long)step * taken(&next_pair)) {
             const long long o = entry(j);
             if (o >= a.n_order) continue;
-            const bool two = o + 1 < a.n_order;
+            const bool two = step == 2 && o + 1 < a.n_order;
             const uint32_t e[2] = {a.order[o], a.order[two ? o + 1 : o]};
             const bool on[2] = {restricted(e[0]), two && restricted(e[1])};
             if (!on[0] && !on[1]) continue;
@@ -2514,15 +2517,29 @@ int stored_kind(const rljsde_plan *p)
     return p->mirror && p->n_order <= kMirrorBlocksPerSm * p->sm_count ? kSoloMirror : kSolo;
 }
 
+// Learned path: runs of kChunk entries, whose blocks mostly share a table set,
+// or single entries where every block can have a warp: the blocks then spread
+// over the SMs, and a shortlisted block does not wait for its half-warp
+// neighbour's column each iteration.  nu_max 100, columns cold, runs of eight in
+// pairs / single: nothing sent back, 32x32 99 / 68 us, 64x64 95 / 73, 160x160 95 /
+// 76; all sent back, 183 / 89, 172 / 95, 160 / 111.
+int learned_run_log(const rljsde_plan *p)
+{
+    return p->n_order <= kStoredWarps * p->sm_count ? 0 : 3;
+}
+static_assert(kChunk == 1 << 3, "the learned path's runs are chunks");
+
 // Shape of a stored-C launch: one CTA per SM, with no more warps than keep
-// its number of rounds (a warp alone on its scheduler iterates faster).
+// its number of rounds (a warp alone on its scheduler iterates faster; the
+// learned path's kinds of blocks take all).
 void stored_shape(const rljsde_plan *p, const int kind, int &warps, int &grid)
 {
     const int most = stored_warps(kind);
     const int per_sm = p->n_order > 0 ? (p->n_order + p->sm_count - 1) / p->sm_count : 1;
     const int rounds = (per_sm + most - 1) / most;
     warps = kind == kLearned ? most : (per_sm + rounds - 1) / rounds;
-    const int want = (p->n_order + warps - 1) / warps;
+    const int share = kind == kLearned ? 1 << learned_run_log(p) : warps;
+    const int want = (p->n_order + share - 1) / share;
     grid = want < p->sm_count ? (want > 0 ? want : 1) : p->sm_count;
 }
 
@@ -2847,10 +2864,12 @@ int rljsde_reconstruct_learned(const rljsde_plan_t *plan, const float *lr, size_
     a.max_missing = max_missing;
     a.use_nu_hat = use_nu_hat;
     a.n_restricted = n_restricted;
-    // shortlist blocks first, then the full loop on the rest
-    // with every table set's Gram matrix stored, both loops read its columns
-    if (plan->n_stored > 0 && plan->n_stored == plan->n_tables)
+    // with every table set's Gram matrix stored, both loops read its columns, in one launch
+    if (plan->n_stored > 0 && plan->n_stored == plan->n_tables) {
+        a.run_log = learned_run_log(plan);
         return launch_stored(plan, a, kLearned, (cudaStream_t)stream);
+    }
+    // shortlist blocks first, then the full loop on the rest
     int st = launch_mode(plan, a, 1, plan->learned_warps, plan->learned_minb, (cudaStream_t)stream);
     if (st == RLJSDE_OK) st = launch_mode(plan, a, 2, 4, 0, (cudaStream_t)stream);
     return st;
