@@ -2505,16 +2505,26 @@ StoredFn stored_fn(const rljsde_plan *p, const int kind, const bool trace)
 
 // Which stored-C kernel a plan's blocks take.  Reading column -uv as the
 // mirror of column uv halves the distinct columns but costs a branch and some
-// ten instructions an iteration: it pays while the columns come from HBM or a
-// cold L2, that is with few blocks.  Measured (mirrored / plain, 4x4-LR tile,
-// nu_max 100): 64x64 60 / 87 us, 128x128 77 / 104, 192x192 146 / 187, 256x256
-// (27 blocks per SM) 287 / 296, 384x384 543 / 517, 1024x1024 3164 / 2824.
-constexpr int kMirrorBlocksPerSm = 27;
+// ten instructions an iteration, and its eight warps an SM make the blocks more
+// rounds than the plain loop's twelve do.  It pays where the columns come from
+// HBM or a cold L2, with few blocks, and takes no more rounds: up to 8 blocks
+// an SM, and 13 to 16.  Measured (mirrored / plain, nu_max 100, cold columns, 4x4-
+// and 16x16-LR tile): 64x64 85 / 97 and 90 / 105 us, 128x128 95 / 109 and 105 /
+// 124, 160x160 (11 an SM) 147 / 115 and 162 / 140, 192x192 (16) 150 / 163 and
+// 164 / 195, 208x208 (18) 207 / 179 and 222 / 208, 256x256 (27) 265 / 248 and 277 /
+// 279.
+constexpr int kMirrorBlocksPerSm = 16;
+int blocks_per_sm(const rljsde_plan *p) { return p->n_order > 0 ? (p->n_order + p->sm_count - 1) / p->sm_count : 1; }
+int stored_rounds(const rljsde_plan *p, const int kind)
+{
+    return (blocks_per_sm(p) + stored_warps(kind) - 1) / stored_warps(kind);
+}
 int stored_kind(const rljsde_plan *p)
 {
     if (p->params.precision == 1) return kFp64;
     if (p->params.pairs) return kSoloPairs;
-    return p->mirror && p->n_order <= kMirrorBlocksPerSm * p->sm_count ? kSoloMirror : kSolo;
+    return p->mirror && blocks_per_sm(p) <= kMirrorBlocksPerSm && stored_rounds(p, kSoloMirror) == stored_rounds(p, kSolo)
+               ? kSoloMirror : kSolo;
 }
 
 // Learned path: runs of kChunk entries, whose blocks mostly share a table set,
@@ -2534,10 +2544,8 @@ static_assert(kChunk == 1 << 3, "the learned path's runs are chunks");
 // learned path's kinds of blocks take all).
 void stored_shape(const rljsde_plan *p, const int kind, int &warps, int &grid)
 {
-    const int most = stored_warps(kind);
-    const int per_sm = p->n_order > 0 ? (p->n_order + p->sm_count - 1) / p->sm_count : 1;
-    const int rounds = (per_sm + most - 1) / most;
-    warps = kind == kLearned ? most : (per_sm + rounds - 1) / rounds;
+    const int rounds = stored_rounds(p, kind);
+    warps = kind == kLearned ? stored_warps(kind) : (blocks_per_sm(p) + rounds - 1) / rounds;
     const int share = kind == kLearned ? 1 << learned_run_log(p) : warps;
     const int want = (p->n_order + share - 1) / share;
     grid = want < p->sm_count ? (want > 0 ? want : 1) : p->sm_count;
