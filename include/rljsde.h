@@ -117,9 +117,15 @@ typedef struct {
                              and 3 and for frequency weights with a zero (the
                              FP32 stored loop's state is sqrt(q / D) R, which
                              cannot hold R where q is 0).  FP64 plans store
-                             FP64 matrices (16 MiB per table set) by the same
-                             rule where a single reconstruction earns their
-                             build back, except with pairs.  1 and 3 need
+                             FP64 matrices by the same rule from n_blocks x
+                             nu_max = 250 per table set on, except with pairs;
+                             each table set takes 16 MiB (8 MiB in FP32) and
+                             some 46 us of plan creation.  The two FP64 loops
+                             agree but for FP64 rounding: a score within it
+                             of another may select differently where a whole
+                             image and a part of it take different loops.
+                             Where the memory is gone by the time auto takes
+                             it, nothing is stored.  1 and 3 need
                              the FP32 loop on path 1 and q > 0 wherever it
                              counts (RLJSDE_ERR_UNSUPPORTED otherwise, also
                              when auto would choose path 2 or 3) and fail with

@@ -471,11 +471,13 @@ int create(rljsde_plan **out, int n_images, const uint8_t *const *masks, const i
     // those at least kStoredMinBlocks blocks use (3), or (auto) all, the most
     // used first, within an eighth of the free device memory.
     // FP64 plans store FP64 matrices by the same rule (auto; not for the pair
-    // update, which keeps the factored loop) if one pass earns the build back:
-    // a table set takes about 47 us to build and a block-iteration is at least
-    // 0.18 us (64x64, latency bound) or 0.043 us (256x256) faster; measured,
-    // plan and one pass at nu_max 100, stored / factored: 64x64 6.5 / 6.5 ms,
-    // 128x128 7.1 / 12.1, 256x256 11.3 / 24.1.  Their state is R, so any q will do.
+    // update, which keeps the factored loop) from 250 block-iterations of a pass
+    // per table set on.  A table set takes about 46 us to build (and 16 MiB), a
+    // block-iteration is 0.18 us (64x64, latency bound) to 0.043 us (256x256)
+    // faster: one to five passes at the line earn the build back.  Measured, plan
+    // and one pass, stored / factored: nu_max 100, 64x64 6.4 / 6.5 ms, 128x128 7.0 /
+    // 12.1, 256x256 11.3 / 24.4; nu_max 10, 256x256 8.3 / 5.3 (a pass alone 0.66 /
+    // 2.34).  Their state is R, so any q will do.
     const size_t table_bytes = prm->precision ? kStored64Bytes : kStoredTableBytes;
     const bool can_store =
         prm->precision ? prm->pairs == 0 && total_blocks * prm->nu_max >= 250ll * p->n_tables : foldable;
@@ -502,7 +504,25 @@ int create(rljsde_plan **out, int n_images, const uint8_t *const *masks, const i
         }
     }
 
-    st = upload(&p->d_entries, entries.data(), entries.size() * sizeof(WorkEntry));
+    // The memory of the matrices and of their build is taken before the table
+    // sets are built: where it is gone since the query, auto stores none.
+    double *d_g64 = nullptr;
+    if (p->n_stored) {
+        p->cstore_bytes = table_bytes * (size_t)p->n_stored;
+        if (cudaMalloc(&p->d_cstore, p->cstore_bytes) != cudaSuccess ||
+            cudaMalloc((void **)&d_g64, (size_t)p->n_stored * kStoredBuildDoubles * sizeof(double)) != cudaSuccess) {
+            cudaGetLastError();
+            cudaFree(p->d_cstore);
+            p->d_cstore = nullptr;
+            d_g64 = nullptr;
+            p->cstore_bytes = 0;
+            p->n_stored = p->n_stored_blocks = 0;
+            p->cslot.clear();
+            if (prm->c_supply != 0) st = RLJSDE_ERR_OUT_OF_MEMORY;
+        }
+    }
+
+    if (!st) st = upload(&p->d_entries, entries.data(), entries.size() * sizeof(WorkEntry));
     if (!st) st = upload(&p->d_chunk_table, chunk_table.data(), chunk_table.size() * sizeof(uint32_t));
     if (!st) {
         Consts c;
@@ -564,14 +584,8 @@ int create(rljsde_plan **out, int n_images, const uint8_t *const *masks, const i
             if (!st && !prm->precision) st = upload(&p->d_records_short, host_short.data(), host_short.size());
             if (!st && p->n_stored) {
                 // the Gram matrices (Eq. 14) of the stored table sets, built on the device
-                double *d_g64 = nullptr;
-                p->cstore_bytes = table_bytes * (size_t)p->n_stored;
-                if (cudaMalloc(&p->d_cstore, p->cstore_bytes) != cudaSuccess) {
-                    p->d_cstore = nullptr;
-                    cudaGetLastError();
-                    st = RLJSDE_ERR_OUT_OF_MEMORY;
-                }
-                if (!st) st = upload(&d_g64, g64.data(), g64.size() * sizeof(double));
+                if (cudaMemcpy(d_g64, g64.data(), g64.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
+                    st = RLJSDE_ERR_CUDA;
                 if (!st) st = upload(&p->d_cslot, p->cslot.data(), p->cslot.size() * sizeof(int));
                 if (!st) {
                     std::vector<uint32_t> order;
@@ -587,10 +601,10 @@ int create(rljsde_plan **out, int n_images, const uint8_t *const *masks, const i
                     st = upload(&p->d_order, order.data(), order.size() * sizeof(uint32_t));
                 }
                 if (!st) st = build_stored_c(p, d_g64);
-                cudaFree(d_g64);
             }
         }
     }
+    cudaFree(d_g64);
     if (!st && (p->direct || p->onthefly)) {
         // Direct path and in-kernel tables: q on the device, no host tables.
         std::vector<float> qf(kK);
