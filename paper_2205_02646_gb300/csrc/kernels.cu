@@ -1214,12 +1214,13 @@ __device__ __forceinline__ C2<float> h_of(const C2<float> *om, int k, int t)
     return csub(P, t == 0 ? C2<float>{1, 0} : t == 1 ? ev : t == 2 ? eu : euv);
 }
 
-// State of one half-warp lane: its four candidates, their R, q_k / D_k, and
-// h_t(k) packed by type pairs (t = 0, 1 and t = 2, 3 in the two halves of
-// an f32x2 register): re, im and -im.
+// State of one half-warp lane: its four candidates, their R and q_k / D_k; the
+// factored loop's h_t(k) packed by type pairs (t = 0, 1 and t = 2, 3 in the two
+// halves of an f32x2 register): re, im and -im; the stored loop's place of each
+// candidate in a column (float4, and which half of it).
 struct HalfState {
     int kc[4];
-    int coff[4], ce;                 // stored C: each candidate's float4 in a column, and which half of it
+    int coff[4], ce;
     float2 Rre[2], Rim[2], qd[2];    // slots (0, 1) and (2, 3) packed
     float2 hre[4][2], him[4][2], nhim[4][2];
 };
@@ -1227,7 +1228,8 @@ struct HalfState {
 // Setup of one block for half-warp hb, with the whole warp working on it:
 // the candidates reordered, R^0_k = sum_t conj(h_t(k)) Y_t(k mod 16) with
 // the column DFTs evaluated at the candidates only, then handed to the lanes
-// of half hb, which add h_t(k) and q_k / D_k.
+// of half hb, which add q_k / D_k and what their loop's column needs.
+template <bool STORED>
 __device__ __forceinline__ void shortlist_setup(const Args &a, const RecordShortF32 &rec, C2<float> *scratch,
                                                 const C2<float> *om, const C2<float> *omc, const float *wt,
                                                 const WorkEntry we, const Shortlist &sl, const int lane, const int hb,
@@ -1307,7 +1309,7 @@ __device__ __forceinline__ void shortlist_setup(const Args &a, const RecordShort
 #pragma unroll
         for (int sl4 = 0; sl4 < 4; ++sl4) {
             st.kc[sl4] = kn[sl4];
-            {
+            if constexpr (STORED) {
                 // where the stored-C loop's lanes keep candidate k in a column:
                 // float4 slot_pair * 32 + lane, low or high half
                 const int k1 = kn[sl4] >> 5;
@@ -1316,14 +1318,16 @@ __device__ __forceinline__ void shortlist_setup(const Args &a, const RecordShort
             }
             if (sl4 & 1) { st.Rre[sl4 >> 1].y = Rn[sl4].re; st.Rim[sl4 >> 1].y = Rn[sl4].im; }
             else { st.Rre[sl4 >> 1].x = Rn[sl4].re; st.Rim[sl4 >> 1].x = Rn[sl4].im; }
-            C2<float> hk[4];
+            if constexpr (!STORED) {
+                C2<float> hk[4];
 #pragma unroll
-            for (int t = 0; t < 4; ++t) hk[t] = h_of(om, kn[sl4], t);
+                for (int t = 0; t < 4; ++t) hk[t] = h_of(om, kn[sl4], t);
 #pragma unroll
-            for (int pr = 0; pr < 2; ++pr) {
-                st.hre[sl4][pr] = f2(hk[2 * pr].re, hk[2 * pr + 1].re);
-                st.him[sl4][pr] = f2(hk[2 * pr].im, hk[2 * pr + 1].im);
-                st.nhim[sl4][pr] = f2(-hk[2 * pr].im, -hk[2 * pr + 1].im);
+                for (int pr = 0; pr < 2; ++pr) {
+                    st.hre[sl4][pr] = f2(hk[2 * pr].re, hk[2 * pr + 1].re);
+                    st.him[sl4][pr] = f2(hk[2 * pr].im, hk[2 * pr + 1].im);
+                    st.nhim[sl4][pr] = f2(-hk[2 * pr].im, -hk[2 * pr + 1].im);
+                }
             }
             if (sl4 & 1) st.qd[sl4 >> 1].y = rec.qD[kn[sl4]];
             else st.qd[sl4 >> 1].x = rec.qD[kn[sl4]];
@@ -1343,11 +1347,9 @@ __device__ __forceinline__ void shortlist_pair(const Args &a, const RecordShortF
 {
     const int hb = lane >> 4;
     HalfState st;
-    st.ce = 0;
 #pragma unroll
     for (int sl4 = 0; sl4 < 4; ++sl4) {
         st.kc[sl4] = 0;
-        st.coff[sl4] = 0;
         if (sl4 < 2) st.Rre[sl4] = st.Rim[sl4] = st.qd[sl4] = f2(0.f, 0.f);
 #pragma unroll
         for (int pr = 0; pr < 2; ++pr) st.hre[sl4][pr] = st.him[sl4][pr] = st.nhim[sl4][pr] = f2(0.f, 0.f);
@@ -1357,7 +1359,7 @@ __device__ __forceinline__ void shortlist_pair(const Args &a, const RecordShortF
     for (int b = 0; b < 2; ++b)
         if (on[b]) {
             const Shortlist &sl = a.shortlists[we[b].ord];
-            shortlist_setup(a, rec, scratch, om, omc, wt, we[b], sl, lane, b, st);
+            shortlist_setup<false>(a, rec, scratch, om, omc, wt, we[b], sl, lane, b, st);
             nu[b] = shortlist_iterations(a, sl);
         }
     const int nu_h = hb == 0 ? nu[0] : nu[1];
@@ -1473,7 +1475,7 @@ __device__ __forceinline__ void shortlist_stored(const Args &a, const uint32_t (
         if (on[b]) {
             const Shortlist &sl = a.shortlists[we[b].ord];
             const RecordShortF32 &rec = reinterpret_cast<const RecordShortF32 *>(a.records_short)[a.chunk_table[e[b] / kChunk]];
-            shortlist_setup(a, rec, scratch, om, omc, wt, we[b], sl, lane, b, st);
+            shortlist_setup<true>(a, rec, scratch, om, omc, wt, we[b], sl, lane, b, st);
             nu[b] = shortlist_iterations(a, sl);
         }
     // the stored columns' scaled state R'_k = s_k R_k, s_k = sqrt(q_k / D_k)
@@ -1602,13 +1604,6 @@ template <int MODE> struct Loop<float, MODE> {
             C2<float> Y[8][4];
             initial_projection<float>(a, rec.types, scratch, omc, wt, we, lane, Y);
             greedy_loop_f32<lay_of(MODE), pairs_of(MODE)>(a, rec, om, omc, pt, we, lane, Y);
-        } else if constexpr (learned_of(MODE) == 1) {
-            const Shortlist &sl = a.shortlists[we.ord];
-            if (!(sl.missing <= a.max_missing)) return;
-            if (a.n_restricted != nullptr && lane == 0) atomicAdd(a.n_restricted, 1);
-            const WorkEntry w2[2] = {we, we};
-            const bool on[2] = {true, false};
-            shortlist_pair(a, rec, scratch, om, omc, wt, w2, on, lane);
         } else {
             const Shortlist &sl = a.shortlists[we.ord];
             if (sl.missing <= a.max_missing) return;
@@ -1642,14 +1637,6 @@ template <int MODE> struct Loop<double, MODE> {
         C2<double> Y[8][4];
         initial_projection<double>(a, rec.types, scratch, omc, wt, we, lane, Y);
         greedy_loop<double, lay_of(MODE), pairs_of(MODE)>(a, rec, om, omc, we, lane, Y);
-    }
-    static __device__ __forceinline__ void run_pair(const Args &a, const Record<double> &rec, C2<double> *scratch,
-                                                    const C2<double> *om, const C2<double> *omc,
-                                                    const PairTables &pt, const double *wt, const WorkEntry e0,
-                                                    const WorkEntry e1, const int lane)
-    {
-        if (e0.img >= 0) run(a, rec, scratch, om, omc, pt, wt, e0, lane);
-        if (e1.img >= 0) run(a, rec, scratch, om, omc, pt, wt, e1, lane);
     }
 };
 
@@ -1749,7 +1736,8 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) recurrent_kernel(const Args 
         }
         if (!work) {
             // no block of this chunk in this mode
-        } else if constexpr (learned_of(MODE) == 1 && WARPS * 2 == kChunk) {
+        } else if constexpr (learned_of(MODE) == 1) {
+            static_assert(WARPS * 2 == kChunk, "two blocks a warp");
             const WorkEntry e0 = a.entries[(size_t)c * kChunk + warp];
             const WorkEntry e1 = a.entries[(size_t)c * kChunk + warp + WARPS];
             Loop<T, MODE>::run_pair(a, *slot(s), scratch, om, omc, *pt, wt, e0, e1, lane);
@@ -2437,7 +2425,7 @@ struct Variant {
 const Variant kVariants[] = {
     RLJSDE_VARIANT(float, 4, 3, 0), RLJSDE_VARIANT(float, 4, 4, 0), RLJSDE_VARIANT(float, 8, 2, 0),
     RLJSDE_VARIANT(float, 8, 1, 0), RLJSDE_VARIANT(double, 4, 1, 0), RLJSDE_VARIANT(double, 8, 1, 0),
-    RLJSDE_VARIANT(float, 4, 3, 1), RLJSDE_VARIANT(float, 8, 2, 1), RLJSDE_VARIANT(float, 4, 3, 2),
+    RLJSDE_VARIANT(float, 4, 3, 1), RLJSDE_VARIANT(float, 4, 3, 2),
     RLJSDE_VARIANT(float, 4, 3, 3), RLJSDE_VARIANT(float, 8, 2, 3), RLJSDE_VARIANT(double, 4, 1, 3),
     RLJSDE_VARIANT(float, 4, 3, 4), RLJSDE_VARIANT(float, 8, 2, 4), RLJSDE_VARIANT(double, 4, 1, 4),
     RLJSDE_VARIANT(float, 4, 3, 8), RLJSDE_VARIANT(float, 4, 3, 11), RLJSDE_VARIANT(float, 4, 3, 12),
@@ -2878,7 +2866,7 @@ int rljsde_reconstruct_learned(const rljsde_plan_t *plan, const float *lr, size_
         return launch_stored(plan, a, kLearned, (cudaStream_t)stream);
     }
     // shortlist blocks first, then the full loop on the rest
-    int st = launch_mode(plan, a, 1, plan->learned_warps, plan->learned_minb, (cudaStream_t)stream);
+    int st = launch_mode(plan, a, 1, 4, 3, (cudaStream_t)stream);
     if (st == RLJSDE_OK) st = launch_mode(plan, a, 2, 4, 0, (cudaStream_t)stream);
     return st;
 }
@@ -2908,9 +2896,8 @@ int rljsde_autotune(rljsde_plan_t *plan, const float *lr, size_t lr_pitch, float
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess) return RLJSDE_ERR_CUDA;
     if (cudaEventCreate(&e1) != cudaSuccess) { cudaEventDestroy(e0); return RLJSDE_ERR_CUDA; }
-    const int keep_w = plan->warps, keep_c = plan->ctas_per_sm;
     float best_ms = 1e30f;
-    int best_w = keep_w, best_c = keep_c, st = RLJSDE_OK;
+    int best_w = plan->warps, best_c = plan->ctas_per_sm, st = RLJSDE_OK;
     const int shapes[][2] = {{4, 1}, {4, 2}, {4, 3}, {4, 4}, {8, 1}, {8, 2}};
     for (const auto &sh : shapes) {
         if (plan->direct || plan->onthefly) break;
@@ -2937,7 +2924,6 @@ int rljsde_autotune(rljsde_plan_t *plan, const float *lr, size_t lr_pitch, float
     if (warps_out) *warps_out = plan->warps;
     if (ctas_out) *ctas_out = plan->ctas_per_sm;
     if (ms_out) *ms_out = best_ms < 1e29f ? best_ms : 0.f;
-    (void)keep_w; (void)keep_c;
     return st;
 }
 
