@@ -1067,7 +1067,7 @@ __device__ __forceinline__ void stored_block(const Args &a, const float4 *cs, co
     // the last iteration, which updates nothing, is peeled: with the column
     // loads and the update under a condition the loop spilled (1024x1024, nu_max
     // 100: 2.82 -> 2.67 ms).  The mirrored loop has registers to spare and is
-    // faster with the condition (64x64 82 against 88 us).
+    // faster with the condition (64x64, columns cold: 82 against 88 us).
     for (int it = 0; it < (MIRROR ? last + 1 : last); ++it) {
         const bool more = !MIRROR || it < last;
         const int bk = stored_argmax(R, lane);
@@ -1816,10 +1816,11 @@ enum StoredKind { kSolo, kSoloMirror, kSoloPairs, kLearned, kFp64 };
 // Warps per CTA (one CTA per SM).  Twelve is three per scheduler at 168
 // registers: the loop is bound by the latency of its own instructions (issue
 // active 52 %, ALU and FMA pipes 42 %, no memory unit above 58 %), and the
-// third warp is worth 13 % over eight warps at 222 registers (1024x1024, nu_max
-// 100: 2.82 against 3.24 ms); sixteen at 128 registers spill (8.3 ms, 3.4 ms
-// with the column loaded in two halves).  The mirrored loop runs where blocks
-// are few and keeps eight and no spills (64x64: 60 against 64 us).
+// third warp is worth 17 % over eight (1024x1024, nu_max 100: 2.66 against 3.12
+// ms); sixteen at 128 registers spill (4.3 ms and more however the column is
+// split).  Three-quarter and quarter layouts hold the loop in 163 registers;
+// the general one spills 28 B, the pair update of that layout 8 B.  The mirrored
+// loop runs where blocks are few and keeps eight and no spills.
 constexpr int stored_warps(const int kind) { return kind == kSoloMirror || kind == kFp64 ? 8 : kStoredWarps; }
 
 template <int LAY, int KIND, bool TRACE>
@@ -2190,7 +2191,7 @@ __global__ void __launch_bounds__(kFlyWarps * 32, 2) onthefly_kernel(const Args 
 // exactly the negative of entry n, so one lookup serves four candidates.  The
 // loop over the window branches to code specialised on the aperture.  Bound by
 // issue: about 11 instructions per candidate and measurement (20 before).
-// 96x64 HR, 15 apertures, nu_max 100: 19.4 -> 6.0 ms.
+// 96x64 HR, 15 apertures, nu_max 100: 19.4 -> 6.2 ms.
 constexpr int kDirectWarps = 4;
 struct DirectSmem {
     float4 x[256];                        // w r (re, im), aperture code, weight
